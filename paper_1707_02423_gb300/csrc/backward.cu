@@ -1280,7 +1280,7 @@ __global__ void __launch_bounds__(NT, 1) bwd_res_kernel(CallArgs a, int n_cta, i
       slot = 7 + eg;
     } else if (level == kClassWarp) {
       grp = Group{t & 31, 32, -1, nullptr, nullptr};
-      region = smem + (size_t)(t >> 5) * cc.z_wrp;
+      region = smem + warp_region_at(t >> 5, cc);
       slot = 15 + (t >> 5);
     }
     const size_t ro = (size_t)(region - smem);

@@ -1523,7 +1523,7 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
       slot = 7 + eg;
     } else if (level == kClassWarp) {
       grp = Group{t & 31, 32, -1, nullptr, nullptr};
-      region = smem + (size_t)(t >> 5) * cc.z_wrp;
+      region = smem + warp_region_at(t >> 5, cc);
       slot = 15 + (t >> 5);
     }
     const uint32_t count = single ? 1u : n[level];

@@ -149,6 +149,16 @@ CF_HD size_t group_region(int cls, const ClassCfg& c) {
                                          : c.z_cta);
 }
 
+// Byte offset of warp w's region in the CTA's shared memory.  The warps of an
+// eighth group share that group's region: with 768 threads three regions of
+// 9,376 bytes take 28,128 of an eighth's 28,160, so regions laid out in one
+// run over the CTA would start inside the eighth before theirs, whose group
+// may still be at work on a larger pair.
+CF_HD size_t warp_region_at(int w, const ClassCfg& c) {
+  const int per = c.nt / 256;  // warps of an eighth group
+  return (size_t)(w / per) * c.z_8th + (size_t)(w % per) * c.z_wrp;
+}
+
 // Orientation of a pair that fits both ways: the column graph's lists live in
 // each thread's registers (its first two neighbours) and a column with more
 // than two neighbours makes its lane run extra work while the rest of its warp
