@@ -527,7 +527,7 @@ def make_step(name, dev, tune_cache=None, bwd_tune=0):
     # kernels per forward call: the three plan kernels, the persistent forward
     # and, under a cluster tune, the cluster-tier kernel; per adjoint call: the
     # three plan kernels, the accumulator reset, the adjoint and the scatter
-    n_fwd = 4 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
+    n_fwd = 5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
         (1 if api.tune_info(tune)["matching"].startswith("ranked, sequential") else 0)
     n_bwd = 3 + 1 + 2 + (1 if w.shared else 2)  # plan, zero, large-pair and resident kernels, scatter
     if name == "dist":  # the C ABI directly, every buffer allocated before the timed region
@@ -630,7 +630,7 @@ def make_query_step(w, pa, pb, omega, d_pairs, ws, tune):
     g = api.Graph(dev)
     with g.capture():
         body()
-    n_fwd = 4 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
+    n_fwd = 5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
         (1 if api.tune_info(tune)["matching"].startswith("ranked, sequential") else 0)
 
     def replay():
@@ -975,7 +975,7 @@ def run_ours(args):
         # per step: the three plan kernels, the persistent forward, the
         # cluster-tier kernel when the tune has one, and the deferred
         # matching steps when the tune defers them
-        "gpu_launches": (4 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + (1 if deferred else 0)) * args.steps,
+        "gpu_launches": (5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + (1 if deferred else 0)) * args.steps,
         "clocks": clk,
         "probes": probes,
         "wall_s_timed_region": t_wall,

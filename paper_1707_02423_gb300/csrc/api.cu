@@ -526,7 +526,7 @@ cf_status cf_similarity(const void* d_pack_a, const void* d_pack_b, const int32_
     // only the queue cursors restart; the plan and the status word stay
     e = cudaMemsetAsync(static_cast<char*>(d_ws) + offsetof(WsHeader, q_next), 0, sizeof(uint32_t) * kNumClasses, st);
     if (e != cudaSuccess) return cuda_fail(e, "queue reset");
-    e = cudaMemsetAsync(static_cast<char*>(d_ws) + offsetof(WsHeader, n_def), 0, 2 * sizeof(uint32_t), st);
+    e = cudaMemsetAsync(static_cast<char*>(d_ws) + offsetof(WsHeader, n_def), 0, 3 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "queue reset");
   } else {
     NvtxRange nv("cfsim/plan");

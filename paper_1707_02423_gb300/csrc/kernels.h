@@ -36,6 +36,7 @@ struct CallArgs {
   int ranked;   // matching policy of resident pairs (ClassCfg::ranked)
   int cluster;  // CTAs per cluster of the cluster tier, 0 = none
   int opt_unstaged;  // optimal matching: skip the shared-memory slot pool (CF_FLAG_OPT_UNSTAGED)
+  int n_cta;         // CTAs the forward's team tier can use (set by launch_plan)
   int pp_streams;    // the plain per-pair form: streams its launches are spread over (0/1: the caller's)
 };
 

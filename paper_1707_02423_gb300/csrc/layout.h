@@ -224,12 +224,15 @@ CF_HD Shape classify(int na, int nb, int ea, int eb, const ClassCfg& c, int xa =
   return s;
 }
 
+// Row stride of a global-class pair's matrices: whole 32-byte sectors (bulk
+// copies take multiples of 16 bytes).
+CF_HD int team_ld(int nb) { return (nb + 7) / 8 * 8; }
+
 // Scratch a global-class pair needs: three n_a x n_b float matrices (two
-// iterates and Ehat), row/column norms and the int32 matching state.
+// iterates and E), row/column norms and the int32 matching state.
 CF_HD size_t global_slot_bytes(int na, int nb) {
-  size_t e = (size_t)na * nb;
-  // Ehat, two iterates, norms, matching state, and 64 busy-column sums per row
-  return align_up(4 * (3 * e + 2 * (size_t)(na + nb) + 2 * (size_t)na + nb + 64 + 64 * (size_t)na), kAlign);
+  size_t e = (size_t)na * team_ld(nb);
+  return align_up(4 * (3 * e + 2 * (size_t)(na + nb) + 2 * (size_t)na + nb + 64), kAlign);
 }
 
 // Adjoint checkpoints: X_k is kept for k = 0, S, 2S, ... with S = ceil(sqrt(K)),
@@ -291,6 +294,39 @@ CF_HD int cost_bucket(int64_t cost) {
   return b;
 }
 
+// The forward's teams (pairs of the global class on several CTAs): queue ends
+// of the team levels -- level L has 2^L teams, the last level single CTAs --
+// and the CTAs' barrier words, by parity.
+constexpr int kTeamLevels = 8;
+constexpr int kTeamMaxCta = 208;  // CTAs that can join teams
+struct TeamTable {
+  uint32_t lvl_end[kTeamLevels];
+  uint64_t slot[2][kTeamMaxCta];
+};
+
+// Team level of a global-class pair of (at least) the given cost when n pairs
+// of the class share n_cta CTAs.
+//   - kTeamEntries entries per CTA and iteration: with fewer, the barrier and
+//     the matching's serial steps (one CTA of the team works) weigh more; with
+//     more, the pairs in flight outgrow L2 and a slab's records the shared
+//     memory.  276 pairs of 500-2,000 blocks: 260 ms at 16 K, 162 at 32 K, 117
+//     at 64 K, 102 at 128 K, 97 at 256 K, 318 at 512 K (no longer staged);
+//   - with fewer pairs than CTAs, more CTAs per pair, down to kTeamMin entries.
+// cost = n_a n_b + 2 e_a e_b is about 3.65 n_a n_b for CFGs (1.15 edges per block).
+constexpr int64_t kTeamEntries = 131072;
+constexpr int64_t kTeamMin = 1024;
+constexpr int kTeamRowCost = 320;  // cost counted per row at least
+CF_HD int team_level(int64_t cost, uint32_t n, int n_cta) {
+  const int64_t cells = cost * 20 / 73;
+  int64_t T = cells / kTeamEntries;
+  const int64_t spare = n > 0 ? n_cta / (int64_t)n : 1, most = cells / kTeamMin;
+  if (T < spare) T = spare < most ? spare : most;
+  if (T < 1) T = 1;
+  int L = 0;
+  while (L < kTeamLevels - 1 && 10 * (int64_t)n_cta > 14 * T * ((int64_t)1 << L)) ++L;
+  return L;
+}
+
 // Workspace header (first bytes of the workspace, zeroed at every call).
 struct WsHeader {
   int32_t status;       // first device-side error (cf_status code), 0 = none
@@ -303,13 +339,19 @@ struct WsHeader {
   uint32_t q_bwd_big;      // adjoint work counter (pairs on clusters)
   uint64_t q_opt;          // optimal-matching work counter (64-bit: claimed by compare-and-swap)
   uint64_t bwd_big_need;   // adjoint scratch bytes of the largest cluster- or global-class pair
-  uint32_t hist[kNumClasses][kBuckets];
-  uint32_t cursor[kNumClasses][kBuckets];
+  union {
+    struct {  // the plan's counts and cursors
+      uint32_t hist[kNumClasses][kBuckets];
+      uint32_t cursor[kNumClasses][kBuckets];
+    };
+    TeamTable team;  // after them: lvl_end from plan_scan on, slot in the forward
+  };
   int64_t x_total, m_total;
   // deferred matching steps (matching policy 3): whether the plan found room
   // for the ranked lists, the byte offset of that area in the workspace, the
   // pairs deferred so far and the second kernel's work counter
-  uint32_t defer, n_def, q_def, pad_;
+  uint32_t defer, n_def, q_def;
+  uint32_t team_bar;  // CTAs of the forward that have cleared their barrier words
   uint64_t defer_off;
 };
 

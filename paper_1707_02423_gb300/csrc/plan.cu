@@ -7,7 +7,10 @@
 // offset sums), scan (one CTA: bucket cursors and block offsets), scatter
 // (queue positions and per-pair offsets).  No host round trip, so the whole
 // call can be replayed from a CUDA graph.
+#include <algorithm>
+
 #include "device_common.cuh"
+#include "device_state.h"
 #include "kernels.h"
 
 namespace cfsim {
@@ -68,7 +71,11 @@ __device__ __forceinline__ PairFacts pair_facts(const PlanCtx& c, int p, const C
   f.n_row = s.n_row;
   f.ld = s.ld;
   // per-iteration work: every entry is written once, every edge pair gathered twice
-  f.bucket = cost_bucket((int64_t)f.na * f.nb + 2 * (int64_t)ea * eb);
+  int64_t cost = (int64_t)f.na * f.nb + 2 * (int64_t)ea * eb;
+  // the global class is split over teams by cost: a CTA's shared memory also
+  // limits the rows of its slab (about 2,000)
+  if (f.cls == kClassGlobal && cost < (int64_t)kTeamRowCost * f.na) cost = (int64_t)kTeamRowCost * f.na;
+  f.bucket = cost_bucket(cost);
   return f;
 }
 
@@ -155,6 +162,20 @@ __global__ void __launch_bounds__(kPlanThreads) plan_scan_kernel(CallArgs a, int
       }
       c.hdr->n_class[cls] = pos - start;
     }
+    // team levels of the global class (the queue's first): the queue position
+    // each level ends at.  The table takes the histogram's place.
+    uint32_t end[kTeamLevels] = {}, seen = 0;
+    const uint32_t ng = c.hdr->n_class[kClassGlobal];
+    int level = 0;
+    for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
+      const uint32_t cnt = c.hdr->hist[kClassGlobal][b];
+      if (cnt == 0) continue;
+      const int64_t cost = (b & 1) ? (int64_t)3 << (b / 2) : (int64_t)2 << (b / 2);  // the bucket's smallest
+      level = max(level, team_level(cost, ng, a.n_cta));
+      seen += cnt;
+      for (int L = level; L < kTeamLevels; ++L) end[L] = seen;
+    }
+    for (int L = 0; L < kTeamLevels; ++L) c.hdr->team.lvl_end[L] = end[L];
   }
   // exclusive scan of the per-block offset sums (chunked over the threads)
   const int per = ceil_div(c.nblk, kPlanThreads);
@@ -217,7 +238,12 @@ __global__ void __launch_bounds__(kPlanThreads) plan_scatter_kernel(CallArgs a, 
 
 }  // namespace
 
-cudaError_t launch_plan(const CallArgs& a, const ClassCfg& cc, cudaStream_t s) {
+cudaError_t launch_plan(const CallArgs& args, const ClassCfg& cc, cudaStream_t s) {
+  CallArgs a = args;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  a.n_cta = std::min(std::max(sm_count_of(dev), 1), kTeamMaxCta);
   WsLayout L = ws_layout(a.P);
   plan_count_kernel<<<L.plan_blocks, kPlanThreads, 0, s>>>(a, cc);
   plan_scan_kernel<<<1, kPlanThreads, 0, s>>>(a, cc.ranked);
