@@ -530,8 +530,6 @@ cf_status cf_similarity(const void* d_pack_a, const void* d_pack_b, const int32_
     if (e != cudaSuccess) return cuda_fail(e, "queue reset");
   } else {
     NvtxRange nv("cfsim/plan");
-    e = cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st);
-    if (e != cudaSuccess) return cuda_fail(e, "workspace reset");
     e = launch_plan(a, fwd_class_cfg(tn.variant, a.min_cls, a.ranked, a.cluster), st);
     if (e != cudaSuccess) return cuda_fail(e, "plan launch");
   }
@@ -576,9 +574,7 @@ cf_status cf_match(const void* d_pack_a, const void* d_pack_b, const int32_t* d_
   a.scores = d_scores;
   a.match = d_match;
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st);
-  if (e != cudaSuccess) return cuda_fail(e, "workspace reset");
-  e = launch_plan(a, fwd_class_cfg(0, a.min_cls, a.ranked, 0), st);
+  cudaError_t e = launch_plan(a, fwd_class_cfg(0, a.min_cls, a.ranked, 0), st);
   if (e != cudaSuccess) return cuda_fail(e, "plan launch");
   if (params && params->match_mode == CF_MATCH_OPTIMAL)
     e = launch_match_optimal(a, st);
@@ -660,9 +656,7 @@ cf_status cf_similarity_backward(const void* d_pack_a, const void* d_pack_b, con
   a.grad_omega = d_grad_omega;
   a.cluster = sh.cluster;
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st);
-  if (e != cudaSuccess) return cuda_fail(e, "workspace reset");
-  e = launch_plan(a, sh.cc, st);
+  cudaError_t e = launch_plan(a, sh.cc, st);
   if (e != cudaSuccess) return cuda_fail(e, "plan launch");
   e = launch_backward(a, variant, st);
   if (e != cudaSuccess) return cuda_fail(e, "backward launch");

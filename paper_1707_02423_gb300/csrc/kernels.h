@@ -61,8 +61,10 @@ struct Tune {
 };
 Tune decode_tune(int32_t id);
 
-// a7: device-side plan: validate pairs, classify, cost-order them into the
-// queue, and compute the X / match offsets.
+// a7: device-side plan: clear the workspace header, validate pairs, classify,
+// cost-order them into the queue, and compute the X / match offsets.  Up to
+// kPlanSmall pairs in one launch, more in a memset and three.
+constexpr int kPlanSmall = 2048;
 cudaError_t launch_plan(const CallArgs& a, const ClassCfg& cc, cudaStream_t s);
 
 // a2-a6: the batched persistent forward (or one launch per pair).

@@ -3,10 +3,15 @@
 // buckets per octave) into one queue per class, and compute the output offsets
 // x_off[p] = sum_{q<p} n_a n_b and m_off[p] = sum_{q<p} n_a.
 //
-// Three small launches: count (per-pair class/bucket histogram and per-block
-// offset sums), scan (one CTA: bucket cursors and block offsets), scatter
-// (queue positions and per-pair offsets).  No host round trip, so the whole
-// call can be replayed from a CUDA graph.
+// Up to kPlanSmall pairs: one launch of one CTA (plan_small_kernel), which also
+// clears the workspace header.  More: a memset and three small launches --
+// count (per-pair class/bucket histogram and per-block offset sums), scan (one
+// CTA: bucket cursors and block offsets), scatter (queue positions and per-pair
+// offsets).  No host round trip, so the whole call can be replayed from a CUDA
+// graph.
+//
+// The plan is latency: a call on 28 pairs takes 201 us with the one launch, 216
+// with the memset and the three.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -79,9 +84,10 @@ __device__ __forceinline__ PairFacts pair_facts(const PlanCtx& c, int p, const C
   return f;
 }
 
-// Exclusive block scan of two int64 values (256 threads).
+// Exclusive block scan of two int64 values (NT threads).
+template <int NT>
 __device__ __forceinline__ void block_scan2(int64_t& x, int64_t& m, int64_t& tx, int64_t& tm) {
-  __shared__ int64_t sx[kPlanThreads / 32], sm[kPlanThreads / 32];
+  __shared__ int64_t sx[NT / 32], sm[NT / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int64_t ix = x, im = m;  // inclusive within warp
 #pragma unroll
@@ -102,7 +108,7 @@ __device__ __forceinline__ void block_scan2(int64_t& x, int64_t& m, int64_t& tx,
   tx = 0;
   tm = 0;
 #pragma unroll
-  for (int k = 0; k < kPlanThreads / 32; ++k) {
+  for (int k = 0; k < NT / 32; ++k) {
     if (k < w) {
       bx += sx[k];
       bm += sm[k];
@@ -115,6 +121,145 @@ __device__ __forceinline__ void block_scan2(int64_t& x, int64_t& m, int64_t& tx,
   __syncthreads();
 }
 
+// What the workspace header keeps of a pair, beside its queue place.
+struct PairNeeds {
+  unsigned long long slot, bwd_slot, bwd_big;
+};
+__device__ __forceinline__ PairNeeds pair_needs(const PairFacts& f, const ClassCfg& cc, int K, int F_pad) {
+  const bool large = f.cls == kClassGlobal || f.cls == kClassCluster;  // both use a scratch slot
+  PairNeeds n{};
+  if (large) n.slot = global_slot_bytes(f.na, f.nb);
+  n.bwd_slot = bwd_slot_bytes(f.na, f.nb, f.ea, f.eb, K, F_pad);
+  // the adjoint's per-team slots of pairs not resident in one CTA: the
+  // full-matrix layout of the cluster tier, or the global tier's own
+  if (cc.bwd && large) n.bwd_big = f.cls == kClassCluster ? bwd_res_slot_bytes(f.n_row, f.ld, K) : n.bwd_slot;
+  return n;
+}
+__device__ __forceinline__ void max_needs(WsHeader* h, const PairNeeds& n) {
+  if (n.slot) atomicMax(reinterpret_cast<unsigned long long*>(&h->slot_need), n.slot);
+  if (n.bwd_slot) atomicMax(reinterpret_cast<unsigned long long*>(&h->bwd_slot_need), n.bwd_slot);
+  if (n.bwd_big) atomicMax(reinterpret_cast<unsigned long long*>(&h->bwd_big_need), n.bwd_big);
+}
+
+// The queue order: class by class; within a class, costliest bucket first.
+// hist [class][bucket] (shared) -> the buckets' first positions, in place, and
+// the classes' sizes; the first 512 threads of the CTA work, all must call.
+// (One thread walking the 448 counts in global memory, a load after a store
+// each time, took most of the plan's time.)
+constexpr int kSlots = kNumClasses * kBuckets;
+static_assert(kSlots <= 512 && kBuckets == 64, "one thread per bucket");
+__device__ __forceinline__ void queue_order(uint32_t* hist, uint32_t* n_class) {
+  __shared__ uint32_t part[16];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int cls = t / kBuckets, at = cls * kBuckets + (kBuckets - 1 - t % kBuckets);
+  const uint32_t v = t < kSlots ? hist[at] : 0u;
+  uint32_t s = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += u;
+  }
+  if (w < 16 && lane == 31) part[w] = s;
+  __syncthreads();
+  if (t < kSlots) {
+    uint32_t before = 0;
+    for (int k = 0; k < w; ++k) before += part[k];
+    hist[at] = before + s - v;
+    if (t % kBuckets == 0) n_class[cls] = part[w] + part[w + 1];  // a class is two warps
+  }
+  __syncthreads();
+}
+
+// Team levels of the global class (the queue's first): the queue position
+// each level ends at, from the class's counts (one thread; cnt: per bucket).
+__device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, int n_cta, uint32_t* lvl_end) {
+  uint32_t seen = 0;
+  uint32_t end[kTeamLevels] = {};
+  int level = 0;
+  for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
+    if (cnt[b] == 0) continue;
+    const int64_t cost = (b & 1) ? (int64_t)3 << (b / 2) : (int64_t)2 << (b / 2);  // the bucket's smallest
+    level = max(level, team_level(cost, ng, n_cta));
+    seen += cnt[b];
+#pragma unroll
+    for (int L = 0; L < kTeamLevels; ++L)
+      if (L >= level) end[L] = seen;
+  }
+#pragma unroll
+  for (int L = 0; L < kTeamLevels; ++L) lvl_end[L] = end[L];
+}
+
+// matching policy 3: the deferred-steps area at the end of the workspace, if
+// it fits beside one scratch slot (when any pair needs one)
+__device__ __forceinline__ void defer_area(WsHeader* h, const CallArgs& a, int ranked, int64_t x_total, uint32_t n_large,
+                                           size_t slot_need) {
+  if (ranked != 3) return;
+  const WsLayout L = ws_layout(a.P);
+  const size_t need = defer_bytes(a.P, x_total);
+  const size_t avail = a.ws_bytes > L.scratch ? a.ws_bytes - L.scratch : 0;
+  if (need + (n_large > 0 ? slot_need : 0) <= avail) {
+    h->defer = 1;
+    h->defer_off = (a.ws_bytes - need + kAlign - 1) / kAlign * kAlign;
+  }
+}
+
+// The whole plan of up to kPlanSmall pairs by one CTA: two pairs per thread,
+// counts and cursors in shared memory.
+constexpr int kPlanSmallNT = 1024;
+
+__global__ void __launch_bounds__(kPlanSmallNT) plan_small_kernel(CallArgs a, ClassCfg cc) {
+  constexpr int kPer = kPlanSmall / kPlanSmallNT;
+  __shared__ uint32_t hist[kSlots], s_class[kNumClasses], s_glob[kBuckets];
+  PlanCtx c = plan_ctx(a);
+  const int t = threadIdx.x;
+  for (int i = t; i < (int)(sizeof(WsHeader) / 4); i += kPlanSmallNT) reinterpret_cast<uint32_t*>(c.hdr)[i] = 0u;
+  if (t < kSlots) hist[t] = 0u;
+  __syncthreads();
+  PairFacts f[kPer];
+  int64_t xc = 0, mc = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int p = kPer * t + k;
+    f[k].valid = false;
+    if (p >= c.P) continue;
+    f[k] = pair_facts(c, p, cc);
+    if (!f[k].valid) {
+      set_status(c.hdr, 1 /* CF_ERR_INVALID_ARG */, p);
+      continue;
+    }
+    atomicAdd(&hist[f[k].cls * kBuckets + f[k].bucket], 1u);
+    max_needs(c.hdr, pair_needs(f[k], cc, a.K, c.A.F_pad));
+    xc += (int64_t)f[k].na * f[k].nb;
+    mc += f[k].na;
+  }
+  int64_t tx, tm;
+  block_scan2<kPlanSmallNT>(xc, mc, tx, tm);
+  if (t < kBuckets) s_glob[t] = hist[kClassGlobal * kBuckets + t];
+  __syncthreads();
+  queue_order(hist, s_class);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int p = kPer * t + k;
+    if (p >= c.P) continue;
+    c.x_off[p] = xc;
+    c.m_off[p] = mc;
+    if (!f[k].valid) continue;
+    c.queue[atomicAdd(&hist[f[k].cls * kBuckets + f[k].bucket], 1u)] = (uint32_t)p;
+    xc += (int64_t)f[k].na * f[k].nb;
+    mc += f[k].na;
+  }
+  if (t < kNumClasses) c.hdr->n_class[t] = s_class[t];
+  if (t == 0) {
+    c.hdr->x_total = tx;
+    c.hdr->m_total = tm;
+    c.x_off[c.P] = tx;
+    c.m_off[c.P] = tm;
+    defer_area(c.hdr, a, cc.ranked, tx, s_class[kClassGlobal] + s_class[kClassCluster],
+               (size_t)*reinterpret_cast<volatile uint64_t*>(&c.hdr->slot_need));
+    if (s_class[kClassGlobal] > 0) team_levels(s_glob, s_class[kClassGlobal], a.n_cta, c.hdr->team.lvl_end);
+  }
+}
+
 __global__ void __launch_bounds__(kPlanThreads) plan_count_kernel(CallArgs a, ClassCfg cc) {
   PlanCtx c = plan_ctx(a);
   const int p = blockIdx.x * kPlanThreads + threadIdx.x;
@@ -125,68 +270,42 @@ __global__ void __launch_bounds__(kPlanThreads) plan_count_kernel(CallArgs a, Cl
       set_status(c.hdr, 1 /* CF_ERR_INVALID_ARG */, p);
     } else {
       atomicAdd(&c.hdr->hist[f.cls][f.bucket], 1u);
-      if (f.cls == kClassGlobal || f.cls == kClassCluster)  // both use a scratch slot
-        atomicMax(reinterpret_cast<unsigned long long*>(&c.hdr->slot_need),
-                  (unsigned long long)global_slot_bytes(f.na, f.nb));
-      atomicMax(reinterpret_cast<unsigned long long*>(&c.hdr->bwd_slot_need),
-                (unsigned long long)bwd_slot_bytes(f.na, f.nb, f.ea, f.eb, a.K, c.A.F_pad));
-      // the adjoint's per-team slots of pairs not resident in one CTA: the
-      // full-matrix layout of the cluster tier, or the global tier's own
-      if (cc.bwd && (f.cls == kClassGlobal || f.cls == kClassCluster))
-        atomicMax(reinterpret_cast<unsigned long long*>(&c.hdr->bwd_big_need),
-                  (unsigned long long)(f.cls == kClassCluster ? bwd_res_slot_bytes(f.n_row, f.ld, a.K)
-                                                              : bwd_slot_bytes(f.na, f.nb, f.ea, f.eb, a.K,
-                                                                               c.A.F_pad)));
+      max_needs(c.hdr, pair_needs(f, cc, a.K, c.A.F_pad));
       xc = (int64_t)f.na * f.nb;
       mc = f.na;
     }
   }
   int64_t tx, tm;
-  block_scan2(xc, mc, tx, tm);
+  block_scan2<kPlanThreads>(xc, mc, tx, tm);
   if (threadIdx.x == 0) {
     c.bsum[blockIdx.x] = tx;
     c.bsum[c.nblk + blockIdx.x] = tm;
   }
 }
 
-__global__ void __launch_bounds__(kPlanThreads) plan_scan_kernel(CallArgs a, int ranked) {
+constexpr int kScanNT = 512;
+
+__global__ void __launch_bounds__(kScanNT) plan_scan_kernel(CallArgs a, int ranked) {
+  __shared__ uint32_t hist[kSlots], s_class[kNumClasses], s_glob[kBuckets];
   PlanCtx c = plan_ctx(a);
-  if (threadIdx.x == 0) {
-    // queue order: class by class; within a class, costliest bucket first
-    uint32_t pos = 0;
-    for (int cls = 0; cls < kNumClasses; ++cls) {
-      uint32_t start = pos;
-      for (int b = kBuckets - 1; b >= 0; --b) {
-        c.hdr->cursor[cls][b] = pos;
-        pos += c.hdr->hist[cls][b];
-      }
-      c.hdr->n_class[cls] = pos - start;
-    }
-    // team levels of the global class (the queue's first): the queue position
-    // each level ends at.  The table takes the histogram's place.
-    uint32_t end[kTeamLevels] = {}, seen = 0;
-    const uint32_t ng = c.hdr->n_class[kClassGlobal];
-    int level = 0;
-    for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
-      const uint32_t cnt = c.hdr->hist[kClassGlobal][b];
-      if (cnt == 0) continue;
-      const int64_t cost = (b & 1) ? (int64_t)3 << (b / 2) : (int64_t)2 << (b / 2);  // the bucket's smallest
-      level = max(level, team_level(cost, ng, a.n_cta));
-      seen += cnt;
-      for (int L = level; L < kTeamLevels; ++L) end[L] = seen;
-    }
-    for (int L = 0; L < kTeamLevels; ++L) c.hdr->team.lvl_end[L] = end[L];
-  }
+  const int t = threadIdx.x;
+  if (t < kSlots) hist[t] = reinterpret_cast<const uint32_t*>(c.hdr->hist)[t];
+  __syncthreads();
+  if (t < kBuckets) s_glob[t] = hist[kClassGlobal * kBuckets + t];
+  __syncthreads();
+  queue_order(hist, s_class);
+  if (t < kSlots) reinterpret_cast<uint32_t*>(c.hdr->cursor)[t] = hist[t];
+  if (t < kNumClasses) c.hdr->n_class[t] = s_class[t];
   // exclusive scan of the per-block offset sums (chunked over the threads)
-  const int per = ceil_div(c.nblk, kPlanThreads);
-  const int b0 = threadIdx.x * per, b1 = min(c.nblk, b0 + per);
+  const int per = ceil_div(c.nblk, kScanNT);
+  const int b0 = t * per, b1 = min(c.nblk, b0 + per);
   int64_t sx = 0, sm = 0;
   for (int b = b0; b < b1; ++b) {
     sx += c.bsum[b];
     sm += c.bsum[c.nblk + b];
   }
   int64_t tx, tm;
-  block_scan2(sx, sm, tx, tm);
+  block_scan2<kScanNT>(sx, sm, tx, tm);
   for (int b = b0; b < b1; ++b) {
     int64_t vx = c.bsum[b], vm = c.bsum[c.nblk + b];
     c.bsum[b] = sx;
@@ -194,24 +313,14 @@ __global__ void __launch_bounds__(kPlanThreads) plan_scan_kernel(CallArgs a, int
     sx += vx;
     sm += vm;
   }
-  if (threadIdx.x == 0) {
+  if (t == 0) {
     c.hdr->x_total = tx;
     c.hdr->m_total = tm;
     c.x_off[c.P] = tx;
     c.m_off[c.P] = tm;
-    // matching policy 3: the deferred-steps area at the end of the
-    // workspace, if it fits beside one scratch slot (when any pair needs one)
-    if (ranked == 3) {
-      const WsLayout L = ws_layout(c.P);
-      const size_t need = defer_bytes(c.P, tx);
-      const size_t avail = a.ws_bytes > L.scratch ? a.ws_bytes - L.scratch : 0;
-      const size_t slot =
-          c.hdr->n_class[kClassGlobal] + c.hdr->n_class[kClassCluster] > 0 ? (size_t)c.hdr->slot_need : 0;
-      if (need + slot <= avail) {
-        c.hdr->defer = 1;
-        c.hdr->defer_off = (a.ws_bytes - need + kAlign - 1) / kAlign * kAlign;
-      }
-    }
+    defer_area(c.hdr, a, ranked, tx, s_class[kClassGlobal] + s_class[kClassCluster], (size_t)c.hdr->slot_need);
+    // (the levels' table takes the histogram's place)
+    team_levels(s_glob, s_class[kClassGlobal], a.n_cta, c.hdr->team.lvl_end);
   }
 }
 
@@ -229,7 +338,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_scatter_kernel(CallArgs a, 
     }
   }
   int64_t tx, tm;
-  block_scan2(xc, mc, tx, tm);
+  block_scan2<kPlanThreads>(xc, mc, tx, tm);
   if (p < c.P) {
     c.x_off[p] = c.bsum[blockIdx.x] + xc;
     c.m_off[p] = c.bsum[c.nblk + blockIdx.x] + mc;
@@ -244,9 +353,15 @@ cudaError_t launch_plan(const CallArgs& args, const ClassCfg& cc, cudaStream_t s
   const cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   a.n_cta = std::min(std::max(sm_count_of(dev), 1), kTeamMaxCta);
+  if (a.P <= kPlanSmall) {
+    plan_small_kernel<<<1, kPlanSmallNT, 0, s>>>(a, cc);
+    return cudaGetLastError();
+  }
+  const cudaError_t z = cudaMemsetAsync(a.ws, 0, sizeof(WsHeader), s);
+  if (z != cudaSuccess) return z;
   WsLayout L = ws_layout(a.P);
   plan_count_kernel<<<L.plan_blocks, kPlanThreads, 0, s>>>(a, cc);
-  plan_scan_kernel<<<1, kPlanThreads, 0, s>>>(a, cc.ranked);
+  plan_scan_kernel<<<1, kScanNT, 0, s>>>(a, cc.ranked);
   plan_scatter_kernel<<<L.plan_blocks, kPlanThreads, 0, s>>>(a, cc);
   return cudaGetLastError();
 }
