@@ -1008,12 +1008,14 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
 // to single CTAs: the teams of level L have n >> L CTAs each (all the same
 // number, so that a pair's sums do not depend on the team that takes it).
 // No barrier sits between levels.  A level's pairs go round its teams in snake
-// order, single CTAs pull them.  A team uses the scratch slot of its first CTA;
-// with fewer slots than CTAs, slots are shared out along the grid, and the
-// finest level is the one whose teams all have a slot of their own.
+// order, starting with the CTAs that the level before has left free; single
+// CTAs pull them.  With a slot for every pair, pair q of the queue uses slot q;
+// else a team uses the slot of its first CTA, and with fewer slots than CTAs,
+// slots are shared out along the grid and the finest level is the one whose
+// teams all have a slot of their own.
 //
 // A kernel of its own: 16 consumer warps, the busy columns' warps and the
-// copying warp (104 registers a thread, for the column lists), and nearly all
+// copying warp (96 registers a thread, for the column lists), and nearly all
 // of the shared memory for the ring.
 constexpr int kTeamNT = 32 * (16 + kBusyWarps + 1);
 constexpr int kTeamSmem = 225280;
@@ -1043,7 +1045,8 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
   TeamTable& tab = cx.hdr->team;
   const uint32_t n_team = min(grid, (uint32_t)kTeamMaxCta);
   int finest = kTeamLevels - 1;  // single CTAs
-  if (coop && nslots < grid) {
+  const bool own = n <= nslots;  // a slot for every pair
+  if (coop && !own && nslots < grid) {
     finest = 0;
     while (finest + 1 < kTeamLevels - 1 && (n_team >> (finest + 1)) > 0 &&
            (uint64_t)(n_team >> (finest + 1)) * nslots >= n_team)
@@ -1066,20 +1069,20 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
     }
     __syncthreads();
   }
-  uint32_t beg = 0;
+  uint32_t beg = 0, cum = 0;
   for (int L = coop ? 0 : kTeamLevels - 1; L <= finest; ++L) {
     const uint32_t end = L < finest ? min(n, tab.lvl_end[L]) : n;
     if (end <= beg) continue;
     const bool alone = L == kTeamLevels - 1;
     const uint32_t T = alone ? 1u : max(1u, n_team >> L), teams = alone ? grid : n_team / T;
-    const uint32_t k = b / T, first = k * T;
-    const uint64_t si = nslots >= grid || alone ? first : first * nslots / n_team;
-    if (k >= teams || si >= nslots || !bounds_ok(cx.hdr, (si + 1) * need <= cx.scratch_bytes, kSiteFwdSlot)) {
+    const uint32_t k = b / T, first = k * T, off = cum / T % teams;
+    const uint64_t team_slot = nslots >= grid || alone ? first : first * nslots / n_team;
+    cum += (end - beg) * T;
+    if (k >= teams || (!own && team_slot >= nslots)) {
       beg = end;  // left over by the teams' size, or a single CTA without a slot
       continue;
     }
-    // (bulk copies need 16-byte addresses; a slot has room for the shift)
-    float* slot = reinterpret_cast<float*>(align_up(reinterpret_cast<size_t>(cx.scratch + si * need), 16));
+    const uint32_t order = (k + teams - off) % teams;
     const Team tm{(int)(b - first), (int)T, tab.slot[0] + first, cx.hdr};
     if (t == 0) sh.gen = (uint32_t)L << kTeamGenBits;
     __syncthreads();
@@ -1093,11 +1096,15 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
         pos = beg + (uint32_t)sh.n0;
         __syncthreads();
       } else {
-        pos = beg + m * teams + ((m & 1u) ? teams - 1u - k : k);
+        pos = beg + m * teams + ((m & 1u) ? teams - 1u - order : order);
         if (beg + m * teams >= end) break;
         if (pos >= end) continue;
       }
       if (pos >= end) break;
+      const uint64_t si = own ? pos : team_slot;
+      if (!bounds_ok(cx.hdr, (si + 1) * need <= cx.scratch_bytes, kSiteFwdSlot)) continue;
+      // (bulk copies need 16-byte addresses; a slot has room for the shift)
+      float* slot = reinterpret_cast<float*>(align_up(reinterpret_cast<size_t>(cx.scratch + si * need), 16));
       run_pair_t<kTeamNT>(cx, make_geo(cx, (int)cx.queue[pos], cc), tm, sh, slot, smem, kTeamSmem);
       used = true;
     }

@@ -304,23 +304,27 @@ struct TeamTable {
   uint64_t slot[2][kTeamMaxCta];
 };
 
-// Team level of a global-class pair of (at least) the given cost when n pairs
-// of the class share n_cta CTAs.
+// Team level of a global-class pair of about the given cost among pairs that
+// share n_cta CTAs.
 //   - kTeamEntries entries per CTA and iteration: with fewer, the barrier and
 //     the matching's serial steps (one CTA of the team works) weigh more; with
 //     more, the pairs in flight outgrow L2 and a slab's records the shared
 //     memory.  276 pairs of 500-2,000 blocks: 260 ms at 16 K, 162 at 32 K, 117
 //     at 64 K, 102 at 128 K, 97 at 256 K, 318 at 512 K (no longer staged);
-//   - with fewer pairs than CTAs, more CTAs per pair, down to kTeamMin entries.
-// cost = n_a n_b + 2 e_a e_b is about 3.65 n_a n_b for CFGs (1.15 edges per block).
+//   - while the pairs leave CTAs free, a pair's share of them by its cells, down
+//     to kTeamMin entries, so that all pairs take about as long.
+// cost = n_a n_b + 2 e_a e_b is about 3.65 n_a n_b for CFGs (1.15 edges per
+// block); total: the cost of all pairs of the class.
 constexpr int64_t kTeamEntries = 131072;
 constexpr int64_t kTeamMin = 1024;
 constexpr int kTeamRowCost = 320;  // cost counted per row at least
-CF_HD int team_level(int64_t cost, uint32_t n, int n_cta) {
+CF_HD int team_level(int64_t cost, int64_t total, int n_cta) {
   const int64_t cells = cost * 20 / 73;
   int64_t T = cells / kTeamEntries;
-  const int64_t spare = n > 0 ? n_cta / (int64_t)n : 1, most = cells / kTeamMin;
-  if (T < spare) T = spare < most ? spare : most;
+  const int64_t most = cells / kTeamMin;
+  int64_t share = (int64_t)((double)cost * n_cta / (double)total + 0.5);
+  if (share > most) share = most;
+  if (T < share) T = share;
   if (T < 1) T = 1;
   int L = 0;
   while (L < kTeamLevels - 1 && 10 * (int64_t)n_cta > 14 * T * ((int64_t)1 << L)) ++L;

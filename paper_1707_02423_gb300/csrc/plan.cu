@@ -173,13 +173,16 @@ __device__ __forceinline__ void queue_order(uint32_t* hist, uint32_t* n_class) {
 // Team levels of the global class (the queue's first): the queue position
 // each level ends at, from the class's counts (one thread; cnt: per bucket).
 __device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, int n_cta, uint32_t* lvl_end) {
+  // a bucket's middle cost: 2 to 3, or 3 to 4, times 2^(b / 2)
+  auto mid = [](int b) { return (int64_t)((b & 1) ? 7 : 5) << (b / 2) >> 1; };
+  int64_t total = 0;
+  for (int b = 0; b < kBuckets; ++b) total += cnt[b] * mid(b);
   uint32_t seen = 0;
   uint32_t end[kTeamLevels] = {};
   int level = 0;
   for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
     if (cnt[b] == 0) continue;
-    const int64_t cost = (b & 1) ? (int64_t)3 << (b / 2) : (int64_t)2 << (b / 2);  // the bucket's smallest
-    level = max(level, team_level(cost, ng, n_cta));
+    level = max(level, team_level(mid(b), total, n_cta));
     seen += cnt[b];
 #pragma unroll
     for (int L = 0; L < kTeamLevels; ++L)
