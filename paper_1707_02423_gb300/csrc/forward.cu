@@ -48,6 +48,7 @@ struct Ctx {
   float alpha;
   int K, norm_mode;
   float* X;
+  const float* X_in;  // the caller's matrices (cf_match): only the matching runs
   float* scores;
   int32_t* match;
   const int64_t* x_off;
@@ -376,7 +377,9 @@ __device__ __forceinline__ float greedy_ranked(const Group& grp, const float* X,
 // (int16, nl x len) and then the dead flags (len bytes) over X_K, which the
 // keys replace; the ranked keys rkey (uint32, nl x len) over the Ehat buffer.
 // Returns the score on the group's rank 0; writes match[n_A] (-1 for
-// unmatched rows of A) if given.  A taken NaN entry sets CF_ERR_NUMERIC.
+// unmatched rows of A) if given.  A taken NaN entry sets CF_ERR_NUMERIC.  The
+// steps end, with CF_ERR_NUMERIC, at a key below `least` (a caller's matrix:
+// neither -inf nor NaN is taken; its score is summed over 32 lanes).
 __device__ __forceinline__ uint32_t okey(float x) {
   if (x != x) return 1u;
   if (x == 0.f) x = 0.f;
@@ -390,7 +393,8 @@ __device__ __forceinline__ float okey_value(uint32_t k) {
 template <int R>
 __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int len, const int16_t* rk,
                                                const uint32_t* rkey, unsigned char* dead, int32_t* mo,
-                                               WsHeader* hdr, int pidx) {
+                                               WsHeader* hdr, int pidx, uint32_t least) {
+  const int lanes = least > 1u ? 31 : 0;  // the lanes that take the score's terms in turn
   // (A, B) index of element e of list l: (l, e), or (e, l) when swapped
   auto tie = [&](int l, int e) -> uint32_t {
     return swap ? ((uint32_t)e << 16) | (uint32_t)l : ((uint32_t)l << 16) | (uint32_t)e;
@@ -422,12 +426,15 @@ __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int 
       }
     const uint32_t mk = __reduce_max_sync(0xffffffffu, bk);
     const uint32_t mt = __reduce_min_sync(0xffffffffu, bk == mk ? bt : 0xffffffffu);
-    if (mk == 0u) break;  // no live list (not reached: a live list remains while steps remain)
+    if (mk < least) {  // no live list (not reached: one remains while steps remain), or no key to be taken
+      if (mk && lane == 0 && hdr) set_status(hdr, 6 /* CF_ERR_NUMERIC */, pidx);
+      break;
+    }
     const int hi = (int)(mt >> 16), lo = (int)(mt & 0xffffu);
     const int l = swap ? lo : hi, e = swap ? hi : lo;
+    if (lane == (step & lanes)) sc += okey_value(mk);
     if (lane == 0) {
       dead[e] = 1;
-      sc += okey_value(mk);
       if (mo) mo[hi] = lo;
       if (mk == 1u && hdr) set_status(hdr, 6 /* CF_ERR_NUMERIC */, pidx);
     }
@@ -463,12 +470,14 @@ __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int 
         }
       }
   }
+  if (lanes)
+    for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
   return sc;
 }
 
 __device__ __forceinline__ float greedy_seq(const Group& grp, float* X, int ld, int n_row, int n_col, int tr,
                                             uint32_t* key, uint32_t* rkey, int32_t* mo, WsHeader* hdr, int pidx,
-                                            bool steps = true) {
+                                            bool steps = true, uint32_t least = 1u) {
   const int t = grp.rank, G = grp.size;
   const bool rows = n_col <= n_row;
   const int nl = rows ? n_row : n_col, len = rows ? n_col : n_row;
@@ -505,17 +514,18 @@ __device__ __forceinline__ float greedy_seq(const Group& grp, float* X, int ld, 
     const bool swap = rows == (tr != 0);
     const int Rn = (nl + 31) >> 5;
     if (Rn <= 1)
-      sc = greedy_seq_steps<1>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
+      sc = greedy_seq_steps<1>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
     else if (Rn <= 2)
-      sc = greedy_seq_steps<2>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
+      sc = greedy_seq_steps<2>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
     else if (Rn <= 4)
-      sc = greedy_seq_steps<4>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
+      sc = greedy_seq_steps<4>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
     else
-      sc = greedy_seq_steps<8>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
+      sc = greedy_seq_steps<8>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
   }
   return sc;
 }
 constexpr int kSeqMaxLists = 256;
+constexpr uint32_t kFiniteKey = 0x00800000u;  // okey of the lowest finite float
 
 // Write X_K (resident, possibly transposed, stride ld) to the caller's
 // row-major n_a x n_b output, coalesced on the global side.
@@ -838,6 +848,37 @@ __device__ __forceinline__ void run_pair_s(const Ctx& cx, const Geo& g, const Gr
   grp.sync();
 }
 
+// a5-a6 of a shared-memory-resident pair on the caller's matrix (cf_match): the
+// sequential greedy on ranked lists, as the forward does, on a group of the
+// pair's size.  Region: as run_pair_s's three matrices (key lists, X, keys).
+// What bounds it is the chain of steps, one warp's per pair; small groups keep
+// 16 or more pairs going on an SM.  (One CTA per pair and rounds of rescans,
+// 4,950 pairs of 8-120 blocks: 1.61 ms against 0.535 ms.)
+__device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const Group& grp, unsigned char* region) {
+  const Shape& s = g.s;
+  const int t = grp.rank, ld = s.ld, nn = s.n_row * ld, tot = g.na * g.nb;
+  float* ehb = reinterpret_cast<float*>(region);
+  float* Xs = ehb + nn;
+  float* freeb = Xs + nn;
+  const float* src = cx.X_in + cx.x_off[g.p];
+  int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
+  for (int idx = t; idx < tot; idx += grp.size) {
+    const int ia = idx / g.nb, jb = idx - ia * g.nb;
+    Xs[s.tr ? jb * ld + ia : ia * ld + jb] = src[idx];
+  }
+  grp.sync();
+  float sc;
+  if (max(s.n_row, s.n_col) <= kSeqMaxLists)
+    sc = greedy_seq(grp, Xs, ld, s.n_row, s.n_col, s.tr, reinterpret_cast<uint32_t*>(freeb),
+                    reinterpret_cast<uint32_t*>(ehb), mo, cx.hdr, g.p, true, kFiniteKey);
+  else
+    sc = greedy<int16_t>(grp, Xs, ld, s.n_row, s.n_col, s.tr, reinterpret_cast<int16_t*>(ehb),
+                         reinterpret_cast<int16_t*>(freeb), reinterpret_cast<int16_t*>(freeb) + s.n_col, mo, cx.hdr,
+                         g.p);
+  if (cx.scores && t == 0) cx.scores[g.p] = sc;
+  grp.sync();
+}
+
 }  // namespace
 }  // namespace cfsim
 #include "team.cuh"
@@ -875,6 +916,7 @@ __device__ __forceinline__ bool make_ctx(const CallArgs& a, float* s_om, Ctx& cx
     cx.K = a.K;
     cx.norm_mode = a.norm_mode;
     cx.X = a.X;
+    cx.X_in = a.X_in;
     cx.scores = a.scores;
     cx.match = a.match;
     cx.F = cx.A.F;
@@ -882,12 +924,12 @@ __device__ __forceinline__ bool make_ctx(const CallArgs& a, float* s_om, Ctx& cx
     cx.ranked = a.ranked;
     cx.om = s_om;
     cx.sqom = s_om + kMaxF;
-    *s_ok = (cx.A.F == cx.B.F && cx.A.F_pad == cx.B.F_pad) ? 1 : 0;
+    *s_ok = (a.X_in || (cx.A.F == cx.B.F && cx.A.F_pad == cx.B.F_pad)) ? 1 : 0;
     if (!*s_ok && blockIdx.x == 0) set_status(cx.hdr, 1 /* CF_ERR_INVALID_ARG */, -1);
   }
   __syncthreads();
   if (!*s_ok) return false;
-  if (threadIdx.x < kMaxF) {
+  if (threadIdx.x < kMaxF && !a.X_in) {
     const float v = threadIdx.x < cx.F ? a.omega[threadIdx.x] : 0.f;
     s_om[threadIdx.x] = v;
     s_om[kMaxF + threadIdx.x] = sqrtf(v);
@@ -914,10 +956,13 @@ __host__ __device__ constexpr ClassCfg fwd_cfg(int min_cls = kClassWarp, int ran
                   cluster};
 }
 
-// kSingle: the plain form -- one launch runs exactly one pair, per_pair, on the
-// whole CTA (a global-class pair in scratch slot pp_slot).
-template <int NT, bool kSingle>
+// kMode: the batched forward; the plain form -- one launch runs exactly one
+// pair, per_pair, on the whole CTA (a global-class pair in scratch slot
+// pp_slot); or the matching of the caller's matrices (match_pair_s).
+enum FwdMode { kFwdBatched, kFwdSingle, kFwdMatch };
+template <int NT, int kMode>
 __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_pair, int pp_slot) {
+  constexpr bool kSingle = kMode == kFwdSingle;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) float s_om[2 * kMaxF];  // omega, then sqrt(omega)
   __shared__ Ctx s_cx;
@@ -995,7 +1040,10 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
           break;
         }
       }
-      run_pair_s(cx, g, grp, region, group_region(level, cc));
+      if constexpr (kMode == kFwdMatch)
+        match_pair_s(cx, g, grp, region);
+      else
+        run_pair_s(cx, g, grp, region, group_region(level, cc));
       if (kSingle) break;
     }
     qbase += kSingle ? 0u : n[level];
@@ -1020,6 +1068,8 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
 constexpr int kTeamNT = 32 * (16 + kBusyWarps + 1);
 constexpr int kTeamSmem = 225280;
 
+// kMatch: the matching alone, on the caller's matrices.
+template <bool kMatch>
 __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassCfg cc, int coop) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) float s_om[2 * kMaxF];
@@ -1038,6 +1088,20 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
   const uint32_t b = blockIdx.x, grid = gridDim.x;
   const uint64_t need = cx.hdr->slot_need;
   const uint64_t nslots = need ? cx.scratch_bytes / need : 0;
+  if (kMatch && nslots == 0) {  // the matching alone can do without scratch: a CTA per pair, its state in shared memory
+    const Group cta{t, kTeamNT, 0, sh.redw, sh.redi};
+    int16_t* ms = reinterpret_cast<int16_t*>(smem);
+    for (;;) {
+      __syncthreads();
+      if (t == 0) sh.n0 = (int)atomicAdd(&cx.hdr->q_next[kClassGlobal], 1u);
+      __syncthreads();
+      if ((uint32_t)sh.n0 >= n) return;
+      const Geo g = make_geo(cx, (int)cx.queue[sh.n0], cc);
+      const float sc = greedy<int16_t>(cta, cx.X_in + cx.x_off[g.p], g.nb, g.na, g.nb, 0, ms, ms + g.na,
+                                       ms + g.na + g.nb, cx.match ? cx.match + cx.m_off[g.p] : nullptr, cx.hdr, g.p);
+      if (cx.scores && t == 0) cx.scores[g.p] = sc;
+    }
+  }
   if (nslots == 0) {
     if (b == 0 && t == 0) set_status(cx.hdr, 2 /* CF_ERR_WORKSPACE */, -1);
     return;
@@ -1105,7 +1169,11 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
       if (!bounds_ok(cx.hdr, (si + 1) * need <= cx.scratch_bytes, kSiteFwdSlot)) continue;
       // (bulk copies need 16-byte addresses; a slot has room for the shift)
       float* slot = reinterpret_cast<float*>(align_up(reinterpret_cast<size_t>(cx.scratch + si * need), 16));
-      run_pair_t<kTeamNT>(cx, make_geo(cx, (int)cx.queue[pos], cc), tm, sh, slot, smem, kTeamSmem);
+      const Geo g = make_geo(cx, (int)cx.queue[pos], cc);
+      if constexpr (kMatch)
+        match_pair_t<kTeamNT>(cx, g, tm, sh, slot, cx.X_in + cx.x_off[g.p], slot, smem, kTeamSmem);
+      else
+        run_pair_t<kTeamNT>(cx, g, tm, sh, slot, smem, kTeamSmem);
       used = true;
     }
     if (used) team_leave(tm, sh);
@@ -1393,43 +1461,15 @@ __global__ void __launch_bounds__(kDefNT) match_deferred_kernel(CallArgs a) {
     const int Rn = (nl + 31) >> 5;
     float sc;
     if (Rn <= 1)
-      sc = greedy_seq_steps<1>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
+      sc = greedy_seq_steps<1>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
     else if (Rn <= 2)
-      sc = greedy_seq_steps<2>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
+      sc = greedy_seq_steps<2>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
     else if (Rn <= 4)
-      sc = greedy_seq_steps<4>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
+      sc = greedy_seq_steps<4>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
     else
-      sc = greedy_seq_steps<8>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
+      sc = greedy_seq_steps<8>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
     if (a.scores && lane == 0) a.scores[p] = sc;
     __syncwarp();
-  }
-}
-
-// cf_match on caller-given matrices: one CTA per pair, matching state in
-// shared memory (int16, up to kMaxBlocks rows and columns).
-constexpr int kMatchNT = 512;
-
-__global__ void __launch_bounds__(kMatchNT) match_only_kernel(CallArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ float redf[64];
-  __shared__ int redi[64];
-  const PackView A = load_pack(a.pack_a), B = load_pack(a.pack_b);
-  const WsLayout L = ws_layout(a.P);
-  const int64_t* x_off = reinterpret_cast<const int64_t*>(a.ws + L.x_off);
-  const int64_t* m_off = reinterpret_cast<const int64_t*>(a.ws + L.m_off);
-  WsHeader* hdr = reinterpret_cast<WsHeader*>(a.ws + L.hdr);
-  int16_t* ms = reinterpret_cast<int16_t*>(smem);
-  const Group grp{(int)threadIdx.x, kMatchNT, 0, redf, redi};
-  for (int p = blockIdx.x; p < a.P; p += gridDim.x) {
-    const int pa = a.pairs[2 * p], pb = a.pairs[2 * p + 1];
-    if (pa < 0 || pa >= A.n_cfgs || pb < 0 || pb >= B.n_cfgs) continue;  // recorded by the plan
-    const int na = A.node_off[pa + 1] - A.node_off[pa];
-    const int nb = B.node_off[pb + 1] - B.node_off[pb];
-    const float* X = a.X_in + x_off[p];
-    int32_t* mo = a.match ? a.match + m_off[p] : nullptr;
-    const float sc = greedy<int16_t>(grp, X, nb, na, nb, 0, ms, ms + na, ms + na + nb, mo, hdr, p);
-    if (a.scores && threadIdx.x == 0) a.scores[p] = sc;
-    __syncthreads();
   }
 }
 
@@ -1468,10 +1508,10 @@ cudaError_t fwd_init(int* n_sm) {
   int dev = 0;
   const cudaError_t e = once.run(
       [](int d) {
-        cudaError_t r = cudaFuncSetAttribute(fwd_batched_kernel<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t r = cudaFuncSetAttribute(fwd_batched_kernel<NT, kFwdBatched>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kFwdSmem);
         if (r == cudaSuccess)
-          r = cudaFuncSetAttribute(fwd_batched_kernel<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+          r = cudaFuncSetAttribute(fwd_batched_kernel<NT, kFwdSingle>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kFwdSmem);
         sms[d] = sm_count_of(d);
         return r != cudaSuccess ? r : (sms[d] > 0 ? cudaSuccess : cudaErrorInvalidDevice);
@@ -1497,16 +1537,16 @@ cudaError_t launch_fwd(const CallArgs& a, bool per_pair, cudaStream_t s) {
     e = cudaEventRecord(ps->fork, s);
     for (int k = 0; k < S && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(ps->side[k], ps->fork, 0);
     for (int p = 0; p < a.P && e == cudaSuccess; ++p)
-      fwd_batched_kernel<NT, true><<<1, NT, kFwdSmem, ps->side[p % S]>>>(a, p, p % S);
+      fwd_batched_kernel<NT, kFwdSingle><<<1, NT, kFwdSmem, ps->side[p % S]>>>(a, p, p % S);
     for (int k = 0; k < S && e == cudaSuccess; ++k) {
       e = cudaEventRecord(ps->join[k], ps->side[k]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ps->join[k], 0);
     }
     if (e != cudaSuccess) return e;
   } else if (per_pair) {
-    for (int p = 0; p < a.P; ++p) fwd_batched_kernel<NT, true><<<1, NT, kFwdSmem, s>>>(a, p, 0);
+    for (int p = 0; p < a.P; ++p) fwd_batched_kernel<NT, kFwdSingle><<<1, NT, kFwdSmem, s>>>(a, p, 0);
   } else {
-    fwd_batched_kernel<NT, false><<<n_sm, NT, kFwdSmem, s>>>(a, -1, 0);
+    fwd_batched_kernel<NT, kFwdBatched><<<n_sm, NT, kFwdSmem, s>>>(a, -1, 0);
   }
   return cudaGetLastError();
 }
@@ -1514,13 +1554,14 @@ cudaError_t launch_fwd(const CallArgs& a, bool per_pair, cudaStream_t s) {
 // The team kernel, launched cooperatively (its CTAs wait on one another, so
 // all must be resident); without cooperative launches every global-class pair
 // runs on one CTA.
+template <bool kMatch>
 cudaError_t launch_team(const CallArgs& a, const ClassCfg& cc, cudaStream_t s) {
   static DeviceOnce once;
   static int sms[kMaxDevices], coop[kMaxDevices];
   int dev = 0;
   const cudaError_t e = once.run(
       [](int d) {
-        cudaError_t r = cudaFuncSetAttribute(fwd_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTeamSmem);
+        cudaError_t r = cudaFuncSetAttribute(fwd_team_kernel<kMatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTeamSmem);
         if (cudaDeviceGetAttribute(&coop[d], cudaDevAttrCooperativeLaunch, d) != cudaSuccess) {
           cudaGetLastError();
           coop[d] = 0;
@@ -1540,7 +1581,7 @@ cudaError_t launch_team(const CallArgs& a, const ClassCfg& cc, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = coop[dev] ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, fwd_team_kernel, a, cc, coop[dev]);
+  return cudaLaunchKernelEx(&cfg, fwd_team_kernel<kMatch>, a, cc, coop[dev]);
 }
 
 // Resident clusters of C CTAs of fwd_cluster_kernel<NT>, per device and C
@@ -1621,7 +1662,7 @@ ClassCfg fwd_class_cfg(int v, int min_cls, int ranked, int cluster) {
 
 cudaError_t launch_forward(const CallArgs& a, int variant, bool per_pair, cudaStream_t s) {
   if (!per_pair) {  // the largest pairs first
-    const cudaError_t e = launch_team(a, fwd_class_cfg(variant, a.min_cls, a.ranked, a.cluster), s);
+    const cudaError_t e = launch_team<false>(a, fwd_class_cfg(variant, a.min_cls, a.ranked, a.cluster), s);
     if (e != cudaSuccess) return e;
   }
   if (!per_pair && a.cluster >= 2) {  // the cluster tier first: its pairs are the largest
@@ -1645,21 +1686,30 @@ cudaError_t launch_match_deferred(const CallArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// 16 warps: 16 pairs of a warp each on an SM, 128 registers for the steps.  (768
+// and 1024 threads, 4,950 pairs of 8-120 blocks: the call 752 and 760 us
+// against 731.)
+constexpr int kMatchNT = 512;
+
 cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s) {
+  const ClassCfg cc = match_class_cfg();
+  cudaError_t e = launch_team<true>(a, cc, s);
+  if (e != cudaSuccess) return e;
   static DeviceOnce once;
   static int grid[kMaxDevices];
-  const size_t sm = 2 * (3 * (size_t)kMaxBlocks + 16);
   int dev = 0;
-  const cudaError_t e = once.run(
-      [sm](int d) {
+  e = once.run(
+      [](int d) {
         grid[d] = sm_count_of(d);
-        return cudaFuncSetAttribute(match_only_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        return cudaFuncSetAttribute(fwd_batched_kernel<kMatchNT, kFwdMatch>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kFwdSmem);
       },
       &dev);
   if (e != cudaSuccess) return e;
-  const int g = a.P < grid[dev] ? a.P : grid[dev];
-  if (g > 0) match_only_kernel<<<g, kMatchNT, sm, s>>>(a);
+  fwd_batched_kernel<kMatchNT, kFwdMatch><<<grid[dev], kMatchNT, kFwdSmem, s>>>(a, -1, 0);
   return cudaGetLastError();
 }
+
+ClassCfg match_class_cfg() { return fwd_cfg<kMatchNT>(kClassWarp, 0, 0); }
 
 }  // namespace cfsim

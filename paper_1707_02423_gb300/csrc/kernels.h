@@ -74,7 +74,9 @@ cudaError_t launch_forward(const CallArgs& a, int variant, bool per_pair, cudaSt
 // one warp per pair whose ranked lists the forward left in the workspace.
 cudaError_t launch_match_deferred(const CallArgs& a, cudaStream_t s);
 
-// Greedy matching + score on caller-given matrices.
+// Greedy matching + score on caller-given matrices (the plan must have run with
+// match_class_cfg()).
+ClassCfg match_class_cfg();
 cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s);
 
 // Maximum-weight assignment + score on the matrices a.X_in (the plan must have

@@ -1017,7 +1017,7 @@ constexpr int kKeyPitch = kTop + 1, kColPitch = kTop + 2;
 // is in it).
 __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigned char* dead, int K, uint2* cand,
                                         uint2* out, int lane) {
-  // the lane's three largest live keys (0: none; NaN entries are never taken)
+  // the lane's three largest live keys (0: none; neither NaN nor -inf is ever taken)
   uint32_t m1 = 0, m2 = 0, m3 = 0;
   for (int j0 = lane; j0 < n_col; j0 += 256) {
     float v[8];
@@ -1026,7 +1026,7 @@ __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigne
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int j = j0 + 32 * u;
-      const uint32_t k = j < n_col && !dead[j] && v[u] == v[u] ? okey(v[u]) : 0u;
+      const uint32_t k = j < n_col && !dead[j] && v[u] > -CUDART_INF_F ? okey(v[u]) : 0u;
       const uint32_t a = min(m1, k), b = min(m2, a);
       m1 = max(m1, k);
       m2 = max(m2, a);
@@ -1045,7 +1045,7 @@ __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigne
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int j = j0 + 32 * u + lane;
-      const uint32_t k = j < n_col && !dead[j] && v[u] == v[u] ? okey(v[u]) : 0u;
+      const uint32_t k = j < n_col && !dead[j] && v[u] > -CUDART_INF_F ? okey(v[u]) : 0u;
       const unsigned m = __ballot_sync(0xffffffffu, k >= bound);
       const int at = n + __popc(m & ((1u << lane) - 1u));
       if (k >= bound && at < kCand) cand[at] = make_uint2(k, (uint32_t)j);
@@ -1122,7 +1122,7 @@ __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigne
     uint64_t best = 0;
     for (int j = lane; j < n_col; j += 32) {
       const float v = x[j];
-      if (dead[j] || v != v) continue;
+      if (dead[j] || !(v > -CUDART_INF_F)) continue;
       const uint64_t k = ((uint64_t)okey(v) << 32) | (uint32_t)~j;
       if (k < prev && k > best) best = k;
     }
@@ -1273,7 +1273,7 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
 #pragma unroll
           for (int u = 0; u < 16; ++u) {
             const int j = j0 + 32 * u;
-            if (j < n_col && !dead[j] && v[u] == v[u]) k = max(k, okey(v[u]));
+            if (j < n_col && !dead[j] && v[u] > -CUDART_INF_F) k = max(k, okey(v[u]));
           }
         }
         k = __reduce_max_sync(0xffffffffu, k);
@@ -1294,7 +1294,7 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     }
     const uint64_t mm = block_max2<NW>(sh, vmax, ~vmin, lane, w);
     vmax = (uint32_t)(mm >> 32);
-    if (vmax == 0u) break;  // only NaN entries are left
+    if (vmax == 0u) break;  // no entry is left that can be taken
     vmin = ~(uint32_t)mm;
     const int shift = max(0, 32 - __clz(vmax - vmin) - 8);
 #pragma unroll
@@ -1445,6 +1445,32 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
   return team_sum(tm, sh, sc);
 }
 
+// The matching of a team's pair: X row-major n_row x n_col, written by the team
+// (or the caller's); lists: scratch of two matrices; the slot's state arrays.
+// Ends with a team barrier.
+template <int NT>
+__device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const Team& tm, TeamSh& sh, float* slot,
+                                             const float* X, float* lists, unsigned char* region, int region_bytes) {
+  const int t = threadIdx.x, n_row = g.na, n_col = g.nb;
+  float* rn = slot + 3 * (size_t)n_row * team_ld(n_col);
+  int32_t* ms = reinterpret_cast<int32_t*>(rn + n_row + n_col);
+  int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
+  if (greedy_team_fits(n_row, n_col, NT, region_bytes)) {
+    const float sc = greedy_team<NT>(tm, sh, X, n_row, n_col, reinterpret_cast<uint2*>(lists), ms,
+                                     reinterpret_cast<uint32_t*>(rn), region, mo, g.p);
+    if (cx.scores && tm.c == 0 && t == 0) cx.scores[g.p] = sc;
+    return;
+  }
+  team_sum(tm, sh, 0.f);
+  if (tm.c == 0) {
+    const Group cta{t, NT, 0, sh.redw, sh.redi};
+    const float sc = greedy<int32_t>(cta, X, n_col, n_row, n_col, 0, ms, ms + n_row, ms + n_row + n_col, mo, cx.hdr,
+                                     g.p);
+    if (cx.scores && t == 0) cx.scores[g.p] = sc;
+  }
+  team_sum(tm, sh, 0.f);
+}
+
 // One pair on a team.  Slot: [E | Y | Y'] (n_row rows of ld floats each, ld =
 // n_col rounded up to 8: bulk copies take multiples of 16 bytes), row and
 // column norms, matching state.  E holds the unscaled attribute term: Y_0 = E
@@ -1462,7 +1488,6 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
   float* b0 = eb + E;
   float* b1 = b0 + E;
   float* rn = b1 + E;
-  int32_t* ms = reinterpret_cast<int32_t*>(rn + n_row + n_col);
   const int i0 = (int)((int64_t)n_row * tm.c / tm.T), i1 = (int)((int64_t)n_row * (tm.c + 1) / tm.T);
   const int nr = i1 - i0, nr_max = ceil_div(n_row, tm.T);
 
@@ -1786,21 +1811,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
     team_sum(tm, sh, 0.f);  // the slot is free for the next pair
     return;
   }
-  int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
-  if (greedy_team_fits(n_row, n_col, NT, region_bytes)) {
-    const float sc = greedy_team<NT>(tm, sh, Xn, n_row, n_col, reinterpret_cast<uint2*>(eb), ms,
-                                     reinterpret_cast<uint32_t*>(rn), region, mo, g.p);
-    if (cx.scores && tm.c == 0 && t == 0) cx.scores[g.p] = sc;
-    return;
-  }
-  team_sum(tm, sh, 0.f);
-  if (tm.c == 0) {
-    const Group cta{t, NT, 0, sh.redw, sh.redi};
-    const float sc = greedy<int32_t>(cta, Xn, n_col, n_row, n_col, 0, ms, ms + n_row, ms + n_row + n_col, mo, cx.hdr,
-                                     g.p);
-    if (cx.scores && t == 0) cx.scores[g.p] = sc;
-  }
-  team_sum(tm, sh, 0.f);
+  match_pair_t<NT>(cx, g, tm, sh, slot, Xn, eb, region, region_bytes);
 }
 
 }  // namespace
