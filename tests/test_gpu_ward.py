@@ -84,3 +84,30 @@ def test_profiles_of_all_pair_scores():
     S = api.score_matrix(pairs, res.scores, n)
     assert torch.equal(S, S.T)
     compare_linkage(S.cpu().numpy().astype(np.float64), exact=False)
+
+
+# a warp of rows and one more, the last size with the distances in shared
+# memory and the next, one row per thread and more
+@pytest.mark.parametrize("n,dim", [(31, 3), (32, 33), (33, 64), (237, 16), (238, 17), (239, 15), (240, 1), (300, 40),
+                                   (1024, 9), (1025, 9)])
+def test_sizes(n, dim):
+    compare_linkage(np.random.default_rng(n).random((n, dim)), False)
+
+
+@pytest.mark.parametrize("n", [12, 40, 260])
+def test_tied_distances_in_order(n):
+    # pairs of equal points far apart, in two interleaved orders: the first
+    # n // 2 merges are ties at distance 0, taken by smaller index
+    k = n // 2
+    X = 1024.0 * np.concatenate([np.arange(k), np.arange(k)[::-1]])[:, None]
+    Z = gpu_linkage(X)
+    assert np.array_equal(Z[:k], np.column_stack([np.arange(k), n - 1 - np.arange(k), np.zeros(k), np.full(k, 2)]))
+
+
+def test_no_finite_distance_left():
+    for n in (5, 300):
+        X = np.random.default_rng(n).random((n, 4))
+        X[n // 2] = np.nan
+        with pytest.raises(B.CfsimError) as e:
+            gpu_linkage(X)
+        assert e.value.status == 6  # CF_ERR_NUMERIC
