@@ -63,8 +63,11 @@ __device__ __forceinline__ void grid_at(int t, int n, int N, int& i0, float& a) 
   a = f - (float)i0;
 }
 
+// |x - y|^p.  kP: the exponent where it is 1, 2 or 3 (0: p as given), chosen
+// once per launch, so that the entry loops hold neither the tests nor powf.
+template <int kP>
 __device__ __forceinline__ float powp(float d, float p) {
-  return p == 3.f ? d * d * d : p == 2.f ? d * d : p == 1.f ? d : powf(d, p);
+  return kP == 3 ? d * d * d : kP == 2 ? d * d : kP == 1 ? d : powf(d, p);
 }
 
 // Compensated running sums (Knuth's TwoSum): h + l carries the sum of the
@@ -91,12 +94,13 @@ __device__ __forceinline__ void add_row(Sums6& t, float d2, float d1, float dp, 
 }
 
 // The terms of one entry: x of the interpolated matrix, y of the larger one.
+template <int kP>
 __device__ __forceinline__ void add_entry(float x, float y, float p, float& d2, float& d1, float& dp, float& xx,
                                           float& yy, float& xy) {
   const float d = fabsf(x - y);
   d2 = fmaf(d, d, d2);
   d1 += d;
-  dp += powp(d, p);
+  dp += powp<kP>(d, p);
   xx = fmaf(x, x, xx);
   yy = fmaf(y, y, yy);
   xy = fmaf(x, y, xy);
@@ -104,67 +108,78 @@ __device__ __forceinline__ void add_entry(float x, float y, float p, float& d2, 
 
 // The pair's CSR in the warp's shared memory: sp / lp row pointers of the
 // smaller / larger CFG relative to their first edge, sa / la their edges.
-// Output row r blends source rows i0 and i0 + 1 into R (shared-memory
-// atomics: a column holds at most one entry of each source row, so the two
-// products land on zero in either order with the same float result) and
-// scatters the larger CFG's row r into Y.  The three buffers of each side
-// rotate: the buffers read at row r - 1 are cleared at row r, one warp
-// barrier before row r + 2 writes them again, so each row needs one barrier.
+// Output row r blends source rows i0 and i0 + 1 into R: row i0's products are
+// stored (R is zero and a source row holds a column once), a warp barrier, row
+// i0 + 1's are added; the larger CFG's row r is scattered into Y.  G: the grid
+// of the columns, which is the rows' as well.  The three buffers of each side
+// rotate: the buffers read at row r - 1 are cleared at row r, one warp barrier
+// before row r + 2 writes them again.
+// What bounds it: instructions issued, nearly all of them the row's fixed work.
+// (With the grid computed per row, shared-memory float atomics, which are
+// loops, and the exponent tested per entry, 19,900 pairs of 8-120 blocks took
+// 503 M warp instructions, 0.601 ms; the call 688 us, against 457.)
+template <int kP>
 __device__ __forceinline__ void pair_rows_staged(int n, int N, float p, const int* sp, const CfAdj* sa, const int* lp,
                                                  const CfAdj* la, float* R, float* Y, int ld, const float2* G,
                                                  Sums6& t) {
   const int lane = threadIdx.x & 31;
-  int b = 0;
+  float *Rb = R, *Yb = Y, *Rz = R + 2 * ld, *Yz = Y + 2 * ld;  // this row's, the last row's
+  int g0 = 0;
   for (int r = 0; r < N; ++r) {
-    float* Rb = R + b * ld;
-    float* Yb = Y + b * ld;
-    int i0;
-    float ar;
-    grid_at(r, n, N, i0, ar);
-    const int e0 = sp[i0], e1 = sp[i0 + 1];
-    for (int e = e0 + lane; e < e1; e += 32) {
+    const float2 gr = G[r];
+    const int i0 = __float_as_int(gr.x);
+    const float ar = gr.y;
+    const int e1 = sp[i0 + 1], g1 = lp[r + 1];
+    for (int e = sp[i0] + lane; e < e1; e += 32) {
       const CfAdj x = sa[e];
-      atomicAdd(Rb + x.nbr, (1.f - ar) * x.w);
+      Rb[x.nbr] = (1.f - ar) * x.w;
     }
-    if (ar != 0.f) {
-      const int f1 = sp[i0 + 2];
-      for (int e = e1 + lane; e < f1; e += 32) {
-        const CfAdj x = sa[e];
-        atomicAdd(Rb + x.nbr, ar * x.w);
-      }
-    }
-    const int g0 = lp[r], g1 = lp[r + 1];
     for (int e = g0 + lane; e < g1; e += 32) {
       const CfAdj y = la[e];
       Yb[y.nbr] = y.w;
     }
+    g0 = g1;
     __syncwarp();
+    if (ar != 0.f) {
+      const int f1 = sp[i0 + 2];
+      for (int e = e1 + lane; e < f1; e += 32) {
+        const CfAdj x = sa[e];
+        Rb[x.nbr] += __fmul_rn(ar, x.w);
+      }
+      __syncwarp();
+    }
     float d2 = 0.f, d1 = 0.f, dp = 0.f, xx = 0.f, yy = 0.f, xy = 0.f;
     for (int c = lane; c < N; c += 32) {
       const float2 g = G[c];
       const int j0 = __float_as_int(g.x);
       const float bc = g.y;
       const float x = bc != 0.f ? fmaf(bc, Rb[j0 + 1], (1.f - bc) * Rb[j0]) : Rb[j0];
-      add_entry(x, Yb[c], p, d2, d1, dp, xx, yy, xy);
+      add_entry<kP>(x, Yb[c], p, d2, d1, dp, xx, yy, xy);
+      // clear the buffers of row r - 1 (every reader of them passed this row's barrier; n <= N)
+      Yz[c] = 0.f;
+      if (c < n) Rz[c] = 0.f;
     }
     add_row(t, d2, d1, dp, xx, yy, xy);
-    // clear the buffers of row r - 1 (every reader of them passed this row's barrier)
-    const int bz = b == 0 ? 2 : b - 1;
-    for (int k = lane; k < n; k += 32) R[bz * ld + k] = 0.f;
-    for (int c = lane; c < N; c += 32) Y[bz * ld + c] = 0.f;
-    b = b == 2 ? 0 : b + 1;
+    float* const Rn = Rz == R ? R + 2 * ld : Rz - ld;  // the buffer cleared at the row before
+    float* const Yn = Yz == Y ? Y + 2 * ld : Yz - ld;
+    Rz = Rb;
+    Yz = Yb;
+    Rb = Rn;
+    Yb = Yn;
   }
   // clear the last row's buffers (the one before it was cleared in the loop)
   __syncwarp();
-  const int bl = (N - 1) % 3;
-  for (int k = lane; k < n; k += 32) R[bl * ld + k] = 0.f;
-  for (int c = lane; c < N; c += 32) Y[bl * ld + c] = 0.f;
+  for (int c = lane; c < N; c += 32) {
+    Yz[c] = 0.f;
+    if (c < n) Rz[c] = 0.f;
+  }
   __syncwarp();
 }
 
 // The same rows with the CSR read from global memory and a single buffer of
 // each side (CFGs too large for the staged layout, or pairs with more edges
 // than its edge area holds): three warp barriers per row.
+template <int kP>
 __device__ __forceinline__ void pair_rows_global(int n, int N, float p, const int32_t* sptr, const int32_t* lptr,
                                                  const CfAdj* sadj, const CfAdj* ladj, float* R, float* Y, Sums6& t) {
   const int lane = threadIdx.x & 31;
@@ -194,7 +209,7 @@ __device__ __forceinline__ void pair_rows_global(int n, int N, float p, const in
       float bc;
       grid_at(c, n, N, j0, bc);
       const float x = bc != 0.f ? fmaf(bc, R[j0 + 1], (1.f - bc) * R[j0]) : R[j0];
-      add_entry(x, Y[c], p, d2, d1, dp, xx, yy, xy);
+      add_entry<kP>(x, Y[c], p, d2, d1, dp, xx, yy, xy);
     }
     add_row(t, d2, d1, dp, xx, yy, xy);
     __syncwarp();
@@ -205,6 +220,7 @@ __device__ __forceinline__ void pair_rows_global(int n, int N, float p, const in
   }
 }
 
+template <int kP>
 __global__ void __launch_bounds__(kDistNT) distances_kernel(const void* pack_a, const void* pack_b, const int32_t* pairs,
                                                            int P, float p, float* out, DistWs* ws) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -262,16 +278,16 @@ __global__ void __launch_bounds__(kDistNT) distances_kernel(const void* pack_a, 
       for (int i = lane; i <= N; i += 32) lp[i] = __ldg(L.out_ptr + lb + i) - l0;
       for (int e = lane; e < es; e += 32) ea[e] = ldg_adj(S.out_adj + s0 + e);
       for (int e = lane; e < el; e += 32) ea[es + e] = ldg_adj(L.out_adj + l0 + e);
-      for (int c = lane; c < N; c += 32) {  // read back by the same lane only
+      for (int c = lane; c < N; c += 32) {
         int j0;
         float bc;
         grid_at(c, n, N, j0, bc);
         G[c] = make_float2(__int_as_float(j0), bc);
       }
       __syncwarp();
-      pair_rows_staged(n, N, p, sp, ea, lp, ea + es, R, Y, ld, G, t);
+      pair_rows_staged<kP>(n, N, p, sp, ea, lp, ea + es, R, Y, ld, G, t);
     } else {
-      pair_rows_global(n, N, p, S.out_ptr + sb, L.out_ptr + lb, S.out_adj, L.out_adj, R, Y, t);
+      pair_rows_global<kP>(n, N, p, S.out_ptr + sb, L.out_ptr + lb, S.out_adj, L.out_adj, R, Y, t);
     }
     double v6[6];
 #pragma unroll
@@ -347,7 +363,11 @@ cudaError_t launch_distances(const void* pack_a, const void* pack_b, const int32
   const cudaError_t ie = once.run(
       [](int d) {
         grids[d] = sm_count_of(d);
-        return cudaFuncSetAttribute(distances_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+        cudaError_t r = cudaSuccess;
+        for (const void* f : {(const void*)distances_kernel<0>, (const void*)distances_kernel<1>,
+                              (const void*)distances_kernel<2>, (const void*)distances_kernel<3>})
+          if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+        return r;
       },
       &dev);
   if (ie != cudaSuccess) return ie;
@@ -355,7 +375,13 @@ cudaError_t launch_distances(const void* pack_a, const void* pack_b, const int32
   DistWs* w = static_cast<DistWs*>(ws);
   distances_init_kernel<<<1, 32, 0, s>>>(w);
   const int g = P < grid ? P : grid;
-  if (g > 0) distances_kernel<<<g, kDistNT, kDistSmem, s>>>(pack_a, pack_b, pairs, P, p, out, w);
+  if (g > 0) {
+    const auto kernel = p == 3.f   ? distances_kernel<3>
+                        : p == 2.f ? distances_kernel<2>
+                        : p == 1.f ? distances_kernel<1>
+                                   : distances_kernel<0>;
+    kernel<<<g, kDistNT, kDistSmem, s>>>(pack_a, pack_b, pairs, P, p, out, w);
+  }
   if (scale && P > 0) {
     const size_t blocks = ((size_t)P * kNumDist + 255) / 256;
     distances_scale_kernel<<<(unsigned)(blocks < (size_t)grid ? blocks : (size_t)grid), 256, 0, s>>>(P, out, w);
