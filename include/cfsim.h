@@ -103,7 +103,8 @@ typedef struct cf_params {
   int32_t norm_mode;  /* CF_NORM_FROB (default) or CF_NORM_NONE                   */
   int32_t match_mode; /* CF_MATCH_GREEDY (default) or CF_MATCH_OPTIMAL               */
   uint32_t flags;     /* CF_FLAG_*                                                */
-  int32_t tune;       /* kernel configuration: 0 = built-in default, else an id in
+  int32_t tune;       /* kernel configuration: 0 = built-in default (tune 1, with larger
+                         groups for small batches), else an id in
                          [1, cf_num_tunes()] (cf_autotune picks one)              */
 } cf_params;
 

@@ -351,6 +351,35 @@ void bwd_config(const cf_params* p, int* variant, int* cluster) {
   *cluster = t.cluster;
 }
 
+// Kernel configuration of a forward call.  Tune 0 is tune 1 for batches that
+// fill the chip with small groups.  A batch of few pairs leaves most SMs (and
+// most of an SM) idle under that, and its time is the chain of one pair's
+// sweeps: up to eight pairs per SM run on CTAs of 512 threads (more registers
+// a thread) and on groups as large as let every SM hold its share at once: a
+// whole CTA up to one pair per SM, half a CTA up to four, a quarter up to
+// eight.  Scores, time on 152 SMs with tune 1 / this rule: 28 pairs of 5-20
+// blocks 105 / 61 us, 28 of 40-60 192 / 133, 28 of 100-135 627 / 590; 190 of
+// 8-60 222 / 162, 435 of 8-60 242 / 160, 496 of 60-135 1.09 / 1.03 ms; 780 of
+// 5-20 161 / 104 us, 1,081 of 60-135 2.07 / 2.00 ms.  (At 276 pairs a whole CTA
+// each took 95 us for 5-20 blocks, half a CTA 67; at 780 half a CTA 138 us, a
+// quarter 104, an eighth 89 but no faster than a quarter on larger pairs.)  Past
+// eight pairs per SM the gain goes down to a few per cent.
+// The plan and the batched form go by it (the plain form takes no groups, and
+// keeps tune 1's threads).
+int batch_group(int P) {
+  const int found = device_sm_count(), sms = found > 0 ? found : 152;
+  return P <= sms ? kClassCta : P <= 4 * sms ? kClassHalf : P <= 8 * sms ? kClassQuarter : kClassWarp;
+}
+Tune call_tune(const cf_params* p, int P) {
+  Tune t = decode_tune(p ? p->tune : 0);
+  if (!p || p->tune != 0) return t;
+  const int cls = batch_group(P);
+  if (cls == kClassWarp) return t;
+  t.variant = 1;
+  t.min_cls = cls;
+  return t;
+}
+
 CallArgs base_args(const void* d_pack_a, const void* d_pack_b, const int32_t* d_pairs, int32_t P,
                    const cf_params* params, const float* d_omega, void* d_ws, size_t ws_bytes) {
   CallArgs a{};
@@ -358,7 +387,7 @@ CallArgs base_args(const void* d_pack_a, const void* d_pack_b, const int32_t* d_
   a.pack_b = d_pack_b;
   a.pairs = d_pairs;
   a.P = P;
-  const Tune tn = decode_tune(params ? params->tune : 0);
+  const Tune tn = call_tune(params, P);
   a.min_cls = tn.min_cls;
   a.ranked = tn.ranked;
   a.cluster = 0;
@@ -517,7 +546,7 @@ cf_status cf_similarity(const void* d_pack_a, const void* d_pack_b, const int32_
   a.X = d_X;
   a.scores = optimal ? nullptr : d_scores;
   a.match = optimal ? nullptr : d_match;
-  const Tune tn = decode_tune(params->tune);
+  const Tune tn = call_tune(params, P);
   // the cluster tier only in the batched form, and only where such clusters can be resident
   if (!(params->flags & CF_FLAG_PER_PAIR_LAUNCH) && tn.cluster >= 2) a.cluster = cluster_supported(tn.variant, tn.cluster);
   cudaStream_t st = (cudaStream_t)stream;
@@ -535,7 +564,8 @@ cf_status cf_similarity(const void* d_pack_a, const void* d_pack_b, const int32_
   }
   if (!(params->flags & CF_FLAG_PLAN_ONLY)) {
     NvtxRange nv("cfsim/iterate");
-    e = launch_forward(a, tn.variant, (params->flags & CF_FLAG_PER_PAIR_LAUNCH) != 0, st);
+    const bool per_pair = (params->flags & CF_FLAG_PER_PAIR_LAUNCH) != 0;
+    e = launch_forward(a, per_pair ? decode_tune(params->tune).variant : tn.variant, per_pair, st);
     if (e != cudaSuccess) return cuda_fail(e, "forward launch");
     if (tn.ranked == 3 && (a.scores || a.match)) {  // the deferred steps (a no-op if the plan found no room)
       e = launch_match_deferred(a, st);
