@@ -605,11 +605,8 @@ cf_status cf_match(const void* d_pack_a, const void* d_pack_b, const int32_t* d_
   a.match = d_match;
   cudaStream_t st = (cudaStream_t)stream;
   const bool greedy = !(params && params->match_mode == CF_MATCH_OPTIMAL);
-  if (greedy) {  // match_class_cfg's
-    a.min_cls = kClassWarp;
-    a.ranked = 0;
-  }
-  cudaError_t e = launch_plan(a, greedy ? match_class_cfg() : fwd_class_cfg(0, a.min_cls, a.ranked, 0), st);
+  if (greedy) a.min_cls = batch_group(P);
+  cudaError_t e = launch_plan(a, greedy ? match_class_cfg(a.min_cls) : fwd_class_cfg(0, a.min_cls, a.ranked, 0), st);
   if (e != cudaSuccess) return cuda_fail(e, "plan launch");
   e = greedy ? launch_match_only(a, st) : launch_match_optimal(a, st);
   if (e != cudaSuccess) return cuda_fail(e, "match launch");

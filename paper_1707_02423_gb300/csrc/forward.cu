@@ -377,9 +377,7 @@ __device__ __forceinline__ float greedy_ranked(const Group& grp, const float* X,
 // (int16, nl x len) and then the dead flags (len bytes) over X_K, which the
 // keys replace; the ranked keys rkey (uint32, nl x len) over the Ehat buffer.
 // Returns the score on the group's rank 0; writes match[n_A] (-1 for
-// unmatched rows of A) if given.  A taken NaN entry sets CF_ERR_NUMERIC.  The
-// steps end, with CF_ERR_NUMERIC, at a key below `least` (a caller's matrix:
-// neither -inf nor NaN is taken; its score is summed over 32 lanes).
+// unmatched rows of A) if given.  A taken NaN entry sets CF_ERR_NUMERIC.
 __device__ __forceinline__ uint32_t okey(float x) {
   if (x != x) return 1u;
   if (x == 0.f) x = 0.f;
@@ -393,8 +391,7 @@ __device__ __forceinline__ float okey_value(uint32_t k) {
 template <int R>
 __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int len, const int16_t* rk,
                                                const uint32_t* rkey, unsigned char* dead, int32_t* mo,
-                                               WsHeader* hdr, int pidx, uint32_t least) {
-  const int lanes = least > 1u ? 31 : 0;  // the lanes that take the score's terms in turn
+                                               WsHeader* hdr, int pidx) {
   // (A, B) index of element e of list l: (l, e), or (e, l) when swapped
   auto tie = [&](int l, int e) -> uint32_t {
     return swap ? ((uint32_t)e << 16) | (uint32_t)l : ((uint32_t)l << 16) | (uint32_t)e;
@@ -426,15 +423,12 @@ __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int 
       }
     const uint32_t mk = __reduce_max_sync(0xffffffffu, bk);
     const uint32_t mt = __reduce_min_sync(0xffffffffu, bk == mk ? bt : 0xffffffffu);
-    if (mk < least) {  // no live list (not reached: one remains while steps remain), or no key to be taken
-      if (mk && lane == 0 && hdr) set_status(hdr, 6 /* CF_ERR_NUMERIC */, pidx);
-      break;
-    }
+    if (mk == 0u) break;  // no live list (not reached: a live list remains while steps remain)
     const int hi = (int)(mt >> 16), lo = (int)(mt & 0xffffu);
     const int l = swap ? lo : hi, e = swap ? hi : lo;
-    if (lane == (step & lanes)) sc += okey_value(mk);
     if (lane == 0) {
       dead[e] = 1;
+      sc += okey_value(mk);
       if (mo) mo[hi] = lo;
       if (mk == 1u && hdr) set_status(hdr, 6 /* CF_ERR_NUMERIC */, pidx);
     }
@@ -470,14 +464,12 @@ __device__ __noinline__ float greedy_seq_steps(int lane, bool swap, int nl, int 
         }
       }
   }
-  if (lanes)
-    for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
   return sc;
 }
 
 __device__ __forceinline__ float greedy_seq(const Group& grp, float* X, int ld, int n_row, int n_col, int tr,
                                             uint32_t* key, uint32_t* rkey, int32_t* mo, WsHeader* hdr, int pidx,
-                                            bool steps = true, uint32_t least = 1u) {
+                                            bool steps = true) {
   const int t = grp.rank, G = grp.size;
   const bool rows = n_col <= n_row;
   const int nl = rows ? n_row : n_col, len = rows ? n_col : n_row;
@@ -514,17 +506,16 @@ __device__ __forceinline__ float greedy_seq(const Group& grp, float* X, int ld, 
     const bool swap = rows == (tr != 0);
     const int Rn = (nl + 31) >> 5;
     if (Rn <= 1)
-      sc = greedy_seq_steps<1>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
+      sc = greedy_seq_steps<1>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
     else if (Rn <= 2)
-      sc = greedy_seq_steps<2>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
+      sc = greedy_seq_steps<2>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
     else if (Rn <= 4)
-      sc = greedy_seq_steps<4>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
+      sc = greedy_seq_steps<4>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
     else
-      sc = greedy_seq_steps<8>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx, least);
+      sc = greedy_seq_steps<8>(t, swap, nl, len, rk, rkey, dead, mo, hdr, pidx);
   }
   return sc;
 }
-constexpr int kSeqMaxLists = 256;
 constexpr uint32_t kFiniteKey = 0x00800000u;  // okey of the lowest finite float
 
 // Write X_K (resident, possibly transposed, stride ld) to the caller's
@@ -848,33 +839,156 @@ __device__ __forceinline__ void run_pair_s(const Ctx& cx, const Geo& g, const Gr
   grp.sync();
 }
 
-// a5-a6 of a shared-memory-resident pair on the caller's matrix (cf_match): the
-// sequential greedy on ranked lists, as the forward does, on a group of the
-// pair's size.  Region: as run_pair_s's three matrices (key lists, X, keys).
-// What bounds it is the chain of steps, one warp's per pair; small groups keep
-// 16 or more pairs going on an SM.  (One CTA per pair and rounds of rescans,
-// 4,950 pairs of 8-120 blocks: 1.61 ms against 0.535 ms.)
+// The steps of match_pair_s, on one warp: as greedy_seq_steps, with a list's
+// next key looked up among the keys [element][list] (pitch ld), and the score
+// summed over the lanes.  Neither -inf nor NaN is taken: the steps end there,
+// with CF_ERR_NUMERIC.  by_row: lists are rows of A.
+template <int R>
+__device__ __noinline__ float match_steps(int lane, bool by_row, int nl, int len, int ld, const uint32_t* key,
+                                          const unsigned char* rk, unsigned char* dead, int32_t* mo, WsHeader* hdr,
+                                          int pidx) {
+  // (A, B) index of element e of list l
+  auto tie = [&](int l, int e) -> uint32_t {
+    return by_row ? ((uint32_t)l << 16) | (uint32_t)e : ((uint32_t)e << 16) | (uint32_t)l;
+  };
+  int cur[R], el[R];
+  uint32_t hk[R], ht[R];
+#pragma unroll
+  for (int s = 0; s < R; ++s) {
+    const int l = lane + 32 * s;
+    cur[s] = 0;
+    el[s] = -1;
+    hk[s] = 0u;
+    ht[s] = 0xffffffffu;
+    if (l < nl) {
+      const int e = rk[l * len];
+      el[s] = e;
+      hk[s] = key[e * ld + l];
+      ht[s] = tie(l, e);
+    }
+  }
+  float sc = 0.f;
+  for (int step = 0; step < len; ++step) {
+    uint32_t bk = 0u, bt = 0xffffffffu;
+#pragma unroll
+    for (int s = 0; s < R; ++s)
+      if (hk[s] > bk || (hk[s] == bk && ht[s] < bt)) {
+        bk = hk[s];
+        bt = ht[s];
+      }
+    const uint32_t mk = __reduce_max_sync(0xffffffffu, bk);
+    const uint32_t mt = __reduce_min_sync(0xffffffffu, bk == mk ? bt : 0xffffffffu);
+    if (mk < kFiniteKey) {
+      if (lane == 0 && hdr) set_status(hdr, 6 /* CF_ERR_NUMERIC */, pidx);
+      break;
+    }
+    const int hi = (int)(mt >> 16), lo = (int)(mt & 0xffffu);
+    const int l = by_row ? hi : lo, e = by_row ? lo : hi;
+    if (lane == (step & 31)) sc += okey_value(mk);
+    if (lane == 0) {
+      dead[e] = 1;
+      if (mo) mo[hi] = lo;
+    }
+#pragma unroll
+    for (int s = 0; s < R; ++s)
+      if (lane + 32 * s == l) {  // the taken list
+        el[s] = -1;
+        hk[s] = 0u;
+        ht[s] = 0xffffffffu;
+      }
+    if (step + 1 == len) break;  // every element is taken
+    __syncwarp();                 // dead[e] is visible to the warp
+#pragma unroll
+    for (int s = 0; s < R; ++s)
+      if (el[s] == e) {  // its head died: the next live element of its list
+        const int ll = lane + 32 * s, base = ll * len;
+        int k = cur[s] + 1, v = 0;
+        for (; k < len; ++k) {
+          v = rk[base + k];
+          if (!dead[v]) break;
+        }
+        cur[s] = k;
+        if (k < len) {
+          el[s] = v;
+          hk[s] = key[v * ld + ll];
+          ht[s] = tie(ll, v);
+        } else {  // not reached: a live element remains while steps remain
+          el[s] = -1;
+          hk[s] = 0u;
+          ht[s] = 0xffffffffu;
+        }
+      }
+  }
+  return warp_sum(sc);
+}
+
+// a5-a6 on the caller's matrix (cf_match): the sequential greedy on ranked
+// lists, as the forward does, on a group of the pair's size.  Lists run along
+// the shorter side and their keys lie [element][list], so that the lanes of a
+// warp rank elements of one index in neighbouring lists (no bank conflicts, the
+// same loop bounds); the keys stay in place and the steps look them up, 5 bytes
+// an entry instead of the forward's 12, so that more pairs are at work on an SM.
+// What bounds it is the chain of steps, one warp's per pair.  (4,950 pairs of
+// 8-120 blocks, the kernel: one CTA per pair and rounds of rescans 1.61 ms, the
+// forward's three buffers 0.535; the call 1.81 ms, 0.76 and, as here, 0.57.)
 __device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const Group& grp, unsigned char* region) {
-  const Shape& s = g.s;
-  const int t = grp.rank, ld = s.ld, nn = s.n_row * ld, tot = g.na * g.nb;
-  float* ehb = reinterpret_cast<float*>(region);
-  float* Xs = ehb + nn;
-  float* freeb = Xs + nn;
+  const int t = grp.rank, G = grp.size, na = g.na, nb = g.nb, tot = na * nb;
   const float* src = cx.X_in + cx.x_off[g.p];
   int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
-  for (int idx = t; idx < tot; idx += grp.size) {
-    const int ia = idx / g.nb, jb = idx - ia * g.nb;
-    Xs[s.tr ? jb * ld + ia : ia * ld + jb] = src[idx];
+  const bool by_row = nb <= na;
+  const int nl = by_row ? na : nb, len = by_row ? nb : na;
+  float sc = 0.f;
+  if (nl <= kSeqMaxLists) {
+    const int ld = nl | 1;
+    uint32_t* key = reinterpret_cast<uint32_t*>(region);
+    unsigned char* rk = region + align_up(4 * (size_t)len * ld, 16);
+    unsigned char* dead = rk + nl * len;
+    for (int i0 = t; i0 < tot; i0 += 8 * G) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = i0 + u * G < tot ? __ldg(src + i0 + u * G) : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int idx = i0 + u * G, r = idx / nb, c = idx - r * nb;
+        if (idx < tot) key[by_row ? c * ld + r : r * ld + c] = okey(v[u]);
+      }
+    }
+    if (mo)
+      for (int i = t; i < na; i += G) mo[i] = -1;
+    for (int e = t; e < len; e += G) dead[e] = 0;
+    grp.sync();
+    // rank of element e in list l: elements with a larger key, or an equal key
+    // and a smaller index (keys are >= 1)
+    for (int idx = t; idx < tot; idx += G) {
+      const int e = idx / nl, l = idx - e * nl;
+      const uint32_t* kp = key + l;
+      const uint32_t k = kp[e * ld];
+      int cnt = 0;
+#pragma unroll 4
+      for (int q = 0; q < e; ++q) cnt += kp[q * ld] >= k;
+#pragma unroll 4
+      for (int q = e + 1; q < len; ++q) cnt += kp[q * ld] > k;
+      rk[l * len + cnt] = (unsigned char)e;
+    }
+    grp.sync();
+    if (t < 32) {
+      const int Rn = (nl + 31) >> 5;
+      if (Rn <= 1)
+        sc = match_steps<1>(t, by_row, nl, len, ld, key, rk, dead, mo, cx.hdr, g.p);
+      else if (Rn <= 2)
+        sc = match_steps<2>(t, by_row, nl, len, ld, key, rk, dead, mo, cx.hdr, g.p);
+      else if (Rn <= 4)
+        sc = match_steps<4>(t, by_row, nl, len, ld, key, rk, dead, mo, cx.hdr, g.p);
+      else
+        sc = match_steps<8>(t, by_row, nl, len, ld, key, rk, dead, mo, cx.hdr, g.p);
+    }
+  } else {
+    float* Xs = reinterpret_cast<float*>(region);
+    int16_t* ms = reinterpret_cast<int16_t*>(region + align_up(4 * (size_t)tot, 16));
+    for (int idx = t; idx < tot; idx += G) Xs[idx] = __ldg(src + idx);
+    grp.sync();
+    sc = greedy<int16_t>(grp, Xs, nb, na, nb, 0, ms, ms + na, ms + na + nb, mo, cx.hdr, g.p);
   }
-  grp.sync();
-  float sc;
-  if (max(s.n_row, s.n_col) <= kSeqMaxLists)
-    sc = greedy_seq(grp, Xs, ld, s.n_row, s.n_col, s.tr, reinterpret_cast<uint32_t*>(freeb),
-                    reinterpret_cast<uint32_t*>(ehb), mo, cx.hdr, g.p, true, kFiniteKey);
-  else
-    sc = greedy<int16_t>(grp, Xs, ld, s.n_row, s.n_col, s.tr, reinterpret_cast<int16_t*>(ehb),
-                         reinterpret_cast<int16_t*>(freeb), reinterpret_cast<int16_t*>(freeb) + s.n_col, mo, cx.hdr,
-                         g.p);
   if (cx.scores && t == 0) cx.scores[g.p] = sc;
   grp.sync();
 }
@@ -956,6 +1070,13 @@ __host__ __device__ constexpr ClassCfg fwd_cfg(int min_cls = kClassWarp, int ran
                   cluster};
 }
 
+template <int NT>
+__host__ __device__ constexpr ClassCfg match_cfg(int min_cls) {
+  ClassCfg c = fwd_cfg<NT>(min_cls);
+  c.bwd = 2;
+  return c;
+}
+
 // kMode: the batched forward; the plain form -- one launch runs exactly one
 // pair, per_pair, on the whole CTA (a global-class pair in scratch slot
 // pp_slot); or the matching of the caller's matrices (match_pair_s).
@@ -975,7 +1096,8 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
   if (!make_ctx(a, s_om, s_cx, &s_ok)) return;
   const Ctx& cx = s_cx;
   // the per-pair form keeps every pair on the whole CTA
-  const ClassCfg cc = fwd_cfg<NT>(kSingle ? (int)kClassCta : a.min_cls, a.ranked);
+  const ClassCfg cc = kMode == kFwdMatch ? match_cfg<NT>(a.min_cls)
+                                         : fwd_cfg<NT>(kSingle ? (int)kClassCta : a.min_cls, a.ranked);
   const int t = threadIdx.x;
   const Group cta{t, NT, 0, s_redf[0], s_redi[0]};
 
@@ -1461,13 +1583,13 @@ __global__ void __launch_bounds__(kDefNT) match_deferred_kernel(CallArgs a) {
     const int Rn = (nl + 31) >> 5;
     float sc;
     if (Rn <= 1)
-      sc = greedy_seq_steps<1>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
+      sc = greedy_seq_steps<1>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
     else if (Rn <= 2)
-      sc = greedy_seq_steps<2>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
+      sc = greedy_seq_steps<2>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
     else if (Rn <= 4)
-      sc = greedy_seq_steps<4>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
+      sc = greedy_seq_steps<4>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
     else
-      sc = greedy_seq_steps<8>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p, 1u);
+      sc = greedy_seq_steps<8>(lane, swap, nl, len, rk, rkey, dead, mo, hdr, p);
     if (a.scores && lane == 0) a.scores[p] = sc;
     __syncwarp();
   }
@@ -1692,7 +1814,7 @@ cudaError_t launch_match_deferred(const CallArgs& a, cudaStream_t s) {
 constexpr int kMatchNT = 512;
 
 cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s) {
-  const ClassCfg cc = match_class_cfg();
+  const ClassCfg cc = match_class_cfg(a.min_cls);
   cudaError_t e = launch_team<true>(a, cc, s);
   if (e != cudaSuccess) return e;
   static DeviceOnce once;
@@ -1710,6 +1832,6 @@ cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-ClassCfg match_class_cfg() { return fwd_cfg<kMatchNT>(kClassWarp, 0, 0); }
+ClassCfg match_class_cfg(int min_cls) { return match_cfg<kMatchNT>(min_cls); }
 
 }  // namespace cfsim

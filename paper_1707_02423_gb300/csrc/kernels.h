@@ -75,8 +75,8 @@ cudaError_t launch_forward(const CallArgs& a, int variant, bool per_pair, cudaSt
 cudaError_t launch_match_deferred(const CallArgs& a, cudaStream_t s);
 
 // Greedy matching + score on caller-given matrices (the plan must have run with
-// match_class_cfg()).
-ClassCfg match_class_cfg();
+// match_class_cfg(a.min_cls)).
+ClassCfg match_class_cfg(int min_cls);
 cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s);
 
 // Maximum-weight assignment + score on the matrices a.X_in (the plan must have

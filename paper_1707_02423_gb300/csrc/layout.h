@@ -84,7 +84,8 @@ struct ClassCfg {
                 // with the sequential steps deferred to a second kernel
                 // (one warp per pair) when the workspace has room
   int cluster;  // CTAs per cluster of the cluster tier (0: no cluster tier)
-  int bwd;      // 1: size regions for the adjoint (bwd_resident_bytes), 0: the forward
+  int bwd;      // what regions are sized for: 0 the forward, 1 the adjoint
+                // (bwd_resident_bytes), 2 the matching alone (match_bytes)
 };
 
 // How a pair maps onto a group of G threads.  The "row" graph indexes the
@@ -122,14 +123,25 @@ CF_HD size_t bwd_resident_bytes(int n_row, int ld, int e_row, int n_col, int e_c
   return resident_bytes(n_row, ld, e_row, n_col, e_col) + align_up(8 * (size_t)(e_row + e_col), 16);
 }
 
+// The matching of a caller's matrix: lists along the shorter side, their keys
+// [element][list] (odd pitch) and ranked elements (a byte each), and a flag per
+// element; or, past kSeqMaxLists lists, the matrix and three int16 per line.
+constexpr int kSeqMaxLists = 256;
+CF_HD size_t match_bytes(int na, int nb) {
+  const size_t nl = na > nb ? na : nb, len = na > nb ? nb : na;
+  return nl <= (size_t)kSeqMaxLists ? align_up(4 * len * (nl | 1), 16) + align_up(nl * len + len, 16)
+                                    : align_up(4 * nl * len, 16) + align_up(2 * (size_t)na + 4 * (size_t)nb, 16);
+}
+
 CF_HD size_t pair_bytes(int n_row, int ld, int e_row, int n_col, int e_col, int bwd) {
-  return bwd ? bwd_resident_bytes(n_row, ld, e_row, n_col, e_col) : resident_bytes(n_row, ld, e_row, n_col, e_col);
+  return bwd == 2 ? match_bytes(n_row, n_col)
+         : bwd    ? bwd_resident_bytes(n_row, ld, e_row, n_col, e_col) : resident_bytes(n_row, ld, e_row, n_col, e_col);
 }
 
 CF_HD bool fits(int n_row, int n_col, int e_row, int e_col, int G, size_t region, int* R, int* M, int bwd = 0) {
-  if (n_col > G) return false;
-  *R = G / n_col;
-  *M = ceil_div(n_row, *R);
+  if (n_col > G && bwd != 2) return false;
+  *R = bwd == 2 ? 1 : G / n_col;
+  *M = bwd == 2 ? 1 : ceil_div(n_row, *R);
   return pair_bytes(n_row, pair_ld(n_col), e_row, n_col, e_col, bwd) <= region;
 }
 
