@@ -501,6 +501,11 @@ def timed_steps(step, steps, warmup, flush, stream):
     return [e0.elapsed_time(e1) for e0, e1 in ev]
 
 
+def plan_kernels(n_pairs):
+    """Kernels of the device-side plan of that many pairs."""
+    return 1 if n_pairs <= 2048 else 3
+
+
 def make_step(name, dev, tune_cache=None, bwd_tune=0):
     """The step of one workload through the Python API (kernel configuration
     from the autotuner): returns (step, n_pairs, launches_per_step, tune)."""
@@ -524,12 +529,12 @@ def make_step(name, dev, tune_cache=None, bwd_tune=0):
     out = {"scores": torch.empty(P, dtype=torch.float32, device=dev),
            "match": torch.empty(int(m_off[-1]), dtype=torch.int32, device=dev)}
     tune = pick_tune(pa, pb, pairs_np, omega, tune_cache)
-    # kernels per forward call: the three plan kernels, the persistent forward
-    # and, under a cluster tune, the cluster-tier kernel; per adjoint call: the
-    # three plan kernels, the accumulator reset, the adjoint and the scatter
-    n_fwd = 5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
+    # kernels per forward call: the plan's, the team kernel, the persistent
+    # forward and, under a cluster tune, the cluster-tier kernel; per adjoint
+    # call: the plan's, the accumulator reset, the adjoint and the scatter
+    n_fwd = plan_kernels(P) + 2 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
         (1 if api.tune_info(tune)["matching"].startswith("ranked, sequential") else 0)
-    n_bwd = 3 + 1 + 2 + (1 if w.shared else 2)  # plan, zero, large-pair and resident kernels, scatter
+    n_bwd = plan_kernels(P) + 1 + 2 + (1 if w.shared else 2)  # plan, zero, large-pair and resident kernels, scatter
     if name == "dist":  # the C ABI directly, every buffer allocated before the timed region
         L = B.lib()
         n = C.c_size_t(0)
@@ -630,14 +635,14 @@ def make_query_step(w, pa, pb, omega, d_pairs, ws, tune):
     g = api.Graph(dev)
     with g.capture():
         body()
-    n_fwd = 5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
+    per_call = 2 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + \
         (1 if api.tune_info(tune)["matching"].startswith("ranked, sequential") else 0)
 
     def replay():
         g.launch()
     replay.graph, replay.scores, replay.top, replay.idx = g, scores, top, idx
     replay.win, replay.win_scores, replay.win_match = win, win_scores, win_match
-    return replay, P, 2 * n_fwd + 2
+    return replay, P, plan_kernels(P) + plan_kernels(win.shape[0]) + 2 * per_call + 2
 
 
 def onchip_peak(kind, f_mhz=None):
@@ -725,7 +730,7 @@ def run_workload(args):
         peak, desc, _ = onchip_peak(kind, clocks["sm_mhz"])
         achieved = onchip / (mps * 1e-3) / 1e9
         line["roofline"] = {"bound": "l2" if kind == B.CF_PROBE_L2 else "smem",
-                            "kernel": {"cfg3": "fwd_batched_kernel / fwd_cluster_kernel (global-memory tier)",
+                            "kernel": {"cfg3": "fwd_team_kernel / fwd_cluster_kernel",
                                        "cfg4": "the whole forward + adjoint step",
                                        "cfg5": "the whole query step (forward kernels, top-k, winners' matching)"}[
                                            args.workload],
@@ -936,7 +941,7 @@ def run_ours(args):
                                   "one GPU", "n_cfgs": len(w.cfgs_a), "F": w.F, "K": K_ITERS,
                    "alpha": ALPHA, "l2": "flushed between steps (256 MiB write, outside the step events)",
                    "step": "two CUDA-graph launches: plan (workspace reset + 3 kernels), forward (queue reset + "
-                           "persistent kernel); sum of per-step CUDA events",
+                           "team and persistent kernels); sum of per-step CUDA events",
                    "tune": {**api.tune_info(tune), "autotune_sample_ms": tune_ms}},
         "roofline": {"bound": "smem",
                      "kernel": "fwd_batched_kernel + match_deferred_kernel (the forward graph)" if deferred
@@ -972,10 +977,10 @@ def run_ours(args):
                 "ms_per_step": e2e_s * 1e3,
                 "what": "cf_pack_cfgs (host build + copy) + pinned pair upload + cf_similarity + pinned "
                         "readback of scores and matchings, wall clock"},
-        # per step: the three plan kernels, the persistent forward, the
-        # cluster-tier kernel when the tune has one, and the deferred
+        # per step: the plan's kernels, the team kernel, the persistent forward,
+        # the cluster-tier kernel when the tune has one, and the deferred
         # matching steps when the tune defers them
-        "gpu_launches": (5 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + (1 if deferred else 0)) * args.steps,
+        "gpu_launches": (plan_kernels(P) + 2 + (1 if api.tune_info(tune)["cluster"] >= 2 else 0) + (1 if deferred else 0)) * args.steps,
         "clocks": clk,
         "probes": probes,
         "wall_s_timed_region": t_wall,

@@ -340,7 +340,7 @@ cf_status cf_similarity_noalloc(const void* d_pack_a, const void* d_pack_b, cons
  * makes the forward run the steps itself), and the cluster
  * tier: pairs too large for one CTA split by rows over the 2, 4 or 8 CTAs of
  * a thread-block cluster with the iterates in distributed shared memory (or,
- * with no cluster tier, iterated by one CTA out of L2).  Every tune gives the
+ * with no cluster tier, on teams of CTAs with the iterates in scratch).  Every tune gives the
  * same results up to rounding; only the speed differs. */
 typedef struct cf_tune_info {
   int32_t tune;
@@ -351,8 +351,8 @@ typedef struct cf_tune_info {
                               it fits with the steps deferred to a second
                               kernel                                            */
   int32_t cluster;         /* CTAs per thread-block cluster of the cluster tier
-                              (0: none; pairs too large for one CTA then use the
-                              global-memory tier)                               */
+                              (0: none; pairs too large for one CTA then run on
+                              teams of CTAs, iterates in scratch)               */
 } cf_tune_info;
 int32_t cf_num_tunes(void);
 cf_status cf_tune_describe(int32_t tune, cf_tune_info* out);

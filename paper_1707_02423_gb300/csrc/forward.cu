@@ -1,17 +1,17 @@
 // a2-a7: the batched similarity forward, greedy matching and graph score.
 //
-// One persistent kernel, one 1024-thread CTA per SM, drains six cost-ordered
-// queues (filled by plan.cu), largest work first:
-//   global class:  pairs too large for shared memory; the whole CTA iterates X
-//                  in a scratch slot of the workspace (L2-resident),
+// fwd_team_kernel takes the global class, the pairs too large for one CTA's
+// shared memory, on teams of CTAs (team.cuh).  Then one persistent kernel, one
+// CTA of 1024, 768 or 512 threads per SM, drains five cost-ordered queues
+// (filled by plan.cu), largest work first:
 //   CTA class:     the whole CTA keeps the pair in its 220 KB of shared memory,
-//   half class:    two 512-thread groups (named barriers 5-6) each keep a pair
-//                  in their half of the shared memory,
-//   quarter class: four 256-thread groups (named barriers 1-4) each keep a
-//                  pair in their quarter of the shared memory,
-//   eighth class:  eight 128-thread groups (named barriers 7-14) each keep a
-//                  pair in their eighth of the shared memory,
-//   warp class:    every warp keeps a small pair in its own 1/32 slice.
+//   half class:    two half groups (named barriers 5-6) each keep a pair in
+//                  their half of the shared memory,
+//   quarter class: four quarter groups (named barriers 1-4) each keep a pair
+//                  in their quarter of the shared memory,
+//   eighth class:  eight eighth groups (named barriers 7-14) each keep a pair
+//                  in their eighth of the shared memory,
+//   warp class:    every warp keeps a small pair in its own slice.
 // A group that finds its queue empty goes straight on to the next level's
 // pairs in its own part of the shared memory, so the tail of one class
 // overlaps the next.
@@ -1808,10 +1808,9 @@ cudaError_t launch_match_deferred(const CallArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// 16 warps: 16 pairs of a warp each on an SM, 128 registers for the steps.  (768
-// and 1024 threads, 4,950 pairs of 8-120 blocks: the call 752 and 760 us
-// against 731.)
-constexpr int kMatchNT = 512;
+// 32 warps: 32 pairs of a warp each on an SM.  (4,950 pairs of 8-120 blocks: the
+// call 529 us, 530 with 768 threads, 566 with 512.)
+constexpr int kMatchNT = 1024;
 
 cudaError_t launch_match_only(const CallArgs& a, cudaStream_t s) {
   const ClassCfg cc = match_class_cfg(a.min_cls);

@@ -1,7 +1,7 @@
 // Byte layouts shared by the host runtime and the kernels: the CSR batch pack,
 // the workspace header, and the classification of a pair into an execution
-// class (warp-, CTA- or global-memory-resident).  Plain C++ so that host-only
-// translation units can include it.
+// class (a group of one CTA, a cluster, or a team of CTAs).  Plain C++ so that
+// host-only translation units can include it.
 #pragma once
 
 #include <stddef.h>
@@ -49,10 +49,11 @@ struct PackHeader {
   int64_t off_xdeg;     // uint8 [n_cfgs]: 1 if a block has more than two out- or in-neighbours
 };
 
-// Execution classes of a pair, in queue order: the global-memory tier, the
-// five shared-memory group levels of the persistent kernel (whole CTA, half,
-// quarter and eighth CTA, single warp), and the cluster tier (rows split over
-// the CTAs of a thread-block cluster, iterate in distributed shared memory).
+// Execution classes of a pair, in queue order: the global class (iterates in
+// scratch, rows split over a team of CTAs), the five shared-memory group levels
+// of the persistent kernel (whole CTA, half, quarter and eighth CTA, single
+// warp), and the cluster tier (rows split over the CTAs of a thread-block
+// cluster, iterate in distributed shared memory).
 enum PairClass : int {
   kClassGlobal = 0,
   kClassCta = 1,

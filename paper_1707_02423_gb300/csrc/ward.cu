@@ -172,9 +172,11 @@ __global__ void __launch_bounds__(kWardNT, 1) ward_merge_kernel(int32_t* hdr, fl
     }
   }
   __syncthreads();
-  // with D in shared memory only the warps that own rows go on
-  const int nw = kShared ? (n + 31) >> 5 : kWardNT / 32;
-  if (wid >= nw) return;
+  // with D in shared memory only the warps that own rows go on, and one that
+  // writes the linkage beside them
+  const int nw = kShared ? (n + 31) >> 5 : kWardNT / 32, n_sync = 32 * (kShared ? nw + 1 : nw);
+  if (kShared && wid > nw) return;
+  const bool recorder = t == (kShared ? 32 * nw : 0);
   float rmin[R];
   int rarg[R], nk[R];  // nk 0: retired
 #pragma unroll
@@ -201,12 +203,12 @@ __global__ void __launch_bounds__(kWardNT, 1) ward_merge_kernel(int32_t* hdr, fl
     uint32_t mk = __reduce_min_sync(0xffffffffu, bk);
     uint32_t mp = __reduce_min_sync(0xffffffffu, bk == mk ? bp : 0xffffffffu);
     if (lane == 0) s_best[par][wid] = make_uint2(mk, mp);
-    bar_sync(1, 32 * nw);
+    bar_sync(1, n_sync);
     const uint2 best = lane < nw ? s_best[par][lane] : make_uint2(0xffffffffu, 0xffffffffu);
     mk = __reduce_min_sync(0xffffffffu, best.x);
     mp = __reduce_min_sync(0xffffffffu, best.x == mk ? best.y : 0xffffffffu);
     if (mk >= kInfKey) {  // no finite distance left: NaN or overflow in the points
-      if (t == 0 && atomicCAS(&hdr[0], 0, 6 /* CF_ERR_NUMERIC */) == 0) hdr[1] = step;
+      if (recorder && atomicCAS(&hdr[0], 0, 6 /* CF_ERR_NUMERIC */) == 0) hdr[1] = step;
       return;
     }
     const int a = (int)(mp >> 16), b = (int)(mp & 0xffffu);
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(kWardNT, 1) ward_merge_kernel(int32_t* hdr, fl
         rarg[m] = a;
       }
     }
-    if (t == 0) {
+    if (recorder) {
       if (la >= 0) csize[la] = (uint16_t)ls;
       const int ca = cid[a], cb = cid[b];
       cid[a] = (uint16_t)(n + step);
