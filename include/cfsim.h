@@ -84,7 +84,7 @@ enum {
   CF_FLAG_PLAN_ONLY = 1u << 1,       /* run only the device-side plan of the pair list (cost
                                         order, offsets) into the workspace                  */
   CF_FLAG_REUSE_PLAN = 1u << 2,      /* skip the plan: reuse the one a previous call with the
-                                        same packs, pairs and workspace left there          */
+                                        same packs, pairs, tune and workspace left there    */
   CF_FLAG_OPT_UNSTAGED = 1u << 3,    /* testing: under CF_MATCH_OPTIMAL every matrix is read
                                         from global memory instead of being staged in the
                                         kernel's shared-memory slot pool -- the path a warp
@@ -175,8 +175,9 @@ cf_status cf_out_sizes(const void* h_pack_a, const void* h_pack_b, const int32_t
 /* Workspace bytes cf_similarity / cf_match need for this pair list.  Uses host
  * copies of the packs and pairs only to size; the device calls take device
  * copies.  A larger workspace is fine.  params->tune matters: the tunes whose
- * matching steps are deferred (cf_tune_info.matching 3) need 6 more bytes per
- * X entry, which this adds; size with the tune the call will use. */
+ * matching steps are deferred (cf_tune_info.matching 3; tune 0 for many pairs)
+ * need 6 more bytes per X entry, which this adds; size with the tune the call
+ * will use. */
 cf_status cf_similarity_ws_size(const void* h_pack_a, const void* h_pack_b, const int32_t* h_pairs, int32_t P,
                                 const cf_params* params, size_t* bytes);
 

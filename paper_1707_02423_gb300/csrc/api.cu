@@ -364,6 +364,13 @@ void bwd_config(const cf_params* p, int* variant, int* cluster) {
 // each took 95 us for 5-20 blocks, half a CTA 67; at 780 half a CTA 138 us, a
 // quarter 104, an eighth 89 but no faster than a quarter on larger pairs.)  Past
 // eight pairs per SM the gain goes down to a few per cent.
+// From 32 pairs per SM on, where pairs have 512 entries or more on average, the
+// matching's sequential steps go to the second kernel (as under tune 181, with
+// the same bits): 19,900 pairs of 8-120 blocks 4.93 -> 4.08 ms, of 10-60 2.03 ->
+// 1.88, 4,950 of 80-135 13.0 -> 8.43, of 8-120 1.30 -> 1.27.  (1,770 pairs of
+// 8-120 blocks took 716 us against 579, 19,900 of 5-20 478 against 464: the
+// second kernel has a tail of its own.)  It needs room in the workspace, which
+// cf_similarity_ws_size counts in; without it the forward takes the steps.
 // The plan and the batched form go by it (the plain form takes no groups, and
 // keeps tune 1's threads).
 int batch_group(int P) {
@@ -374,7 +381,14 @@ Tune call_tune(const cf_params* p, int P) {
   Tune t = decode_tune(p ? p->tune : 0);
   if (!p || p->tune != 0) return t;
   const int cls = batch_group(P);
-  if (cls == kClassWarp) return t;
+  if (cls == kClassWarp) {
+    const int found = device_sm_count();
+    if (P >= 32 * (found > 0 ? found : 152) && !(p->flags & CF_FLAG_PER_PAIR_LAUNCH)) {
+      t.ranked = 3;
+      t.defer_auto = 1;
+    }
+    return t;
+  }
   t.variant = 1;
   t.min_cls = cls;
   return t;
@@ -389,6 +403,7 @@ CallArgs base_args(const void* d_pack_a, const void* d_pack_b, const int32_t* d_
   a.P = P;
   const Tune tn = call_tune(params, P);
   a.min_cls = tn.min_cls;
+  a.defer_auto = tn.defer_auto;
   a.ranked = tn.ranked;
   a.cluster = 0;
   if (params) {
@@ -525,7 +540,8 @@ cf_status cf_similarity_ws_size(const void* h_pack_a, const void* h_pack_b, cons
   if (params && (params->flags & CF_FLAG_PER_PAIR_STREAMS) && ng > 0) slots = std::max<int64_t>(slots, kPerPairStreams);
   *bytes = ws_layout(P).fixed_bytes + (size_t)slots * need;
   // matching policy 3: room for every pair's ranked lists (deferred steps)
-  if (params && decode_tune(params->tune).ranked == 3 && !(params->flags & CF_FLAG_PER_PAIR_LAUNCH))
+  const Tune tn = call_tune(params, P);
+  if (tn.ranked == 3 && !(params->flags & CF_FLAG_PER_PAIR_LAUNCH) && (!tn.defer_auto || defer_pays(P, xs)))
     *bytes += defer_bytes(P, xs);
   return ok();
 }

@@ -1020,10 +1020,12 @@ __device__ __forceinline__ bool make_ctx(const CallArgs& a, float* s_om, Ctx& cx
       const uint64_t off = cx.hdr->defer_off;
       const int64_t xt = cx.hdr->x_total;
       cx.scratch_bytes = off > L.scratch ? off - L.scratch : 0;
-      cx.def_rk = reinterpret_cast<int16_t*>(a.ws + off);
-      cx.def_rkey = reinterpret_cast<uint32_t*>(a.ws + off + align_up(2 * (size_t)xt, kAlign));
-      cx.def_list = reinterpret_cast<uint32_t*>(a.ws + off + align_up(2 * (size_t)xt, kAlign) +
-                                                align_up(4 * (size_t)xt, kAlign));
+      if (a.ranked == 3) {  // (a plan used again by a call whose second kernel does not run)
+        cx.def_rk = reinterpret_cast<int16_t*>(a.ws + off);
+        cx.def_rkey = reinterpret_cast<uint32_t*>(a.ws + off + align_up(2 * (size_t)xt, kAlign));
+        cx.def_list = reinterpret_cast<uint32_t*>(a.ws + off + align_up(2 * (size_t)xt, kAlign) +
+                                                  align_up(4 * (size_t)xt, kAlign));
+      }
     }
     cx.pairs = a.pairs;
     cx.alpha = a.alpha;

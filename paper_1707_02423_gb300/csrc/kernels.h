@@ -33,6 +33,7 @@ struct CallArgs {
   float* grad_omega;
   // kernel configuration (the tune of cf_params)
   int min_cls;  // smallest group level of the batched forward
+  int defer_auto;  // the plan defers the matching's steps only where that pays (defer_area)
   int ranked;   // matching policy of resident pairs (ClassCfg::ranked)
   int cluster;  // CTAs per cluster of the cluster tier, 0 = none
   int opt_unstaged;  // optimal matching: skip the shared-memory slot pool (CF_FLAG_OPT_UNSTAGED)
@@ -58,6 +59,7 @@ constexpr int kNumTunes = 240;
 constexpr int kFirstDeferTune = 181;
 struct Tune {
   int variant, min_cls, ranked, cluster;
+  int defer_auto = 0;  // ranked is 3 by the number of pairs (tune 0), not by the caller's tune
 };
 Tune decode_tune(int32_t id);
 

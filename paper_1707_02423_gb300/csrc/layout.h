@@ -380,6 +380,15 @@ CF_HD size_t defer_bytes(int P, int64_t x_total) {
          align_up(4 * (size_t)(P > 0 ? P : 1), kAlign) + kAlign;
 }
 
+// Whether tune 0 defers the matching's steps for a batch of many pairs
+// (call_tune): pairs of kDeferCells entries or more on average, and lists of at
+// most kDeferMost bytes in all.
+constexpr int64_t kDeferCells = 512;
+constexpr size_t kDeferMost = (size_t)2 << 30;
+CF_HD bool defer_pays(int P, int64_t x_total) {
+  return x_total >= kDeferCells * P && defer_bytes(P, x_total) <= kDeferMost;
+}
+
 // Byte offsets of the forward workspace sections for P pairs.
 struct WsLayout {
   size_t hdr, queue, x_off, m_off, bsum, scratch, fixed_bytes;

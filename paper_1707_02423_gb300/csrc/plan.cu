@@ -193,14 +193,21 @@ __device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, in
 }
 
 // matching policy 3: the deferred-steps area at the end of the workspace, if
-// it fits beside one scratch slot (when any pair needs one)
+// it fits beside one scratch slot (when any pair needs one).  Under tune 0 it
+// must leave every slot that the workspace was sized for, and pairs must be
+// large enough on average for the second kernel to pay (kDeferCells).
 __device__ __forceinline__ void defer_area(WsHeader* h, const CallArgs& a, int ranked, int64_t x_total, uint32_t n_large,
                                            size_t slot_need) {
   if (ranked != 3) return;
   const WsLayout L = ws_layout(a.P);
   const size_t need = defer_bytes(a.P, x_total);
   const size_t avail = a.ws_bytes > L.scratch ? a.ws_bytes - L.scratch : 0;
-  if (need + (n_large > 0 ? slot_need : 0) <= avail) {
+  size_t slots = n_large > 0 ? 1 : 0;
+  if (a.defer_auto) {
+    if (!defer_pays(a.P, x_total)) return;
+    slots = n_large < 2u * (uint32_t)a.n_cta ? n_large : 2u * (uint32_t)a.n_cta;
+  }
+  if (need + slots * slot_need <= avail) {
     h->defer = 1;
     h->defer_off = (a.ws_bytes - need + kAlign - 1) / kAlign * kAlign;
   }

@@ -40,3 +40,26 @@ def test_lines(per_sm, more):
             m = mt[r.m_off[p]:r.m_off[p + 1]]
             k = np.flatnonzero(m >= 0)
             assert abs(sc[p] - x[k, m[k]].sum()) <= 1e-5
+
+
+@pytest.mark.parametrize("lo,hi", [(4, 12), (20, 45)])
+def test_large_batch_defers_with_the_same_bits(lo, hi):
+    """32 pairs per SM and more: the steps in the second kernel (pairs large
+    enough, room in the workspace) or in place, with the bits of tune 1."""
+    rng = np.random.default_rng(lo)
+    P = 32 * torch.cuda.get_device_properties(0).multi_processor_count + 5
+    sizes = [int(n) for n in rng.integers(lo, hi, 30)] + [300]
+    cfgs = [structured_cfg(rng, n, 5, 7) for n in sizes]
+    pairs = rng.integers(0, 30, (P, 2)).astype(np.int32)
+    pairs[7] = (30, 3)
+    pairs[8] = (30, 30)
+    pk = api.Pack(cfgs, 8, device=DEV)
+    om = torch.linspace(0.5, 1.5, 8, device=DEV)
+    ref = api.similarity(pk, pk, pairs, om, want_match=True, tune=1)
+    small = api.ws_size(pk, pk, pairs, B.params(tune=1))
+    full = api.ws_size(pk, pk, pairs, B.params())
+    assert (full > small) == (lo == 20)
+    ws = api.Workspace(DEV)
+    for size, flags in ((full, 0), (full, B.CF_FLAG_REUSE_PLAN), (small, 0)):
+        r = api.similarity(pk, pk, pairs, om, want_match=True, ws=ws, ws_bytes=size, flags=flags)
+        assert torch.equal(r.scores, ref.scores) and torch.equal(r.match, ref.match)
