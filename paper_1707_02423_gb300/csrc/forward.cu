@@ -1182,9 +1182,7 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
 // No barrier sits between levels.  A level's pairs go round its teams in snake
 // order, starting with the CTAs that the level before has left free; single
 // CTAs pull them.  With a slot for every pair, pair q of the queue uses slot q;
-// else a team uses the slot of its first CTA, and with fewer slots than CTAs,
-// slots are shared out along the grid and the finest level is the one whose
-// teams all have a slot of their own.
+// else a team has one (team_seat).
 //
 // A kernel of its own: 16 consumer warps, the busy columns' warps and the
 // copying warp (96 registers a thread, for the column lists), and nearly all
@@ -1234,12 +1232,8 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
   const uint32_t n_team = min(grid, (uint32_t)kTeamMaxCta);
   int finest = kTeamLevels - 1;  // single CTAs
   const bool own = n <= nslots;  // a slot for every pair
-  if (coop && !own && nslots < grid) {
-    finest = 0;
-    while (finest + 1 < kTeamLevels - 1 && (n_team >> (finest + 1)) > 0 &&
-           (uint64_t)(n_team >> (finest + 1)) * nslots >= n_team)
-      ++finest;
-  }
+  const bool shared = coop && !own && nslots < grid;
+  if (shared) finest = team_finest(n_team, nslots);
   if (coop && (finest < kTeamLevels - 1 || tab.lvl_end[kTeamLevels - 2] > 0)) {
     // every CTA clears its barrier words before any team uses them
     if (t == 0) {
@@ -1262,15 +1256,14 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
     const uint32_t end = L < finest ? min(n, tab.lvl_end[L]) : n;
     if (end <= beg) continue;
     const bool alone = L == kTeamLevels - 1;
-    const uint32_t T = alone ? 1u : max(1u, n_team >> L), teams = alone ? grid : n_team / T;
-    const uint32_t k = b / T, first = k * T, off = cum / T % teams;
-    const uint64_t team_slot = nslots >= grid || alone ? first : first * nslots / n_team;
+    const TeamSeat seat = team_seat(b, L, n_team, grid, shared, finest);
+    const uint32_t T = seat.T, teams = seat.teams, first = seat.first, off = cum / T % teams;
     cum += (end - beg) * T;
-    if (k >= teams || (!own && team_slot >= nslots)) {
+    if (!seat.in || (!own && seat.slot >= nslots)) {
       beg = end;  // left over by the teams' size, or a single CTA without a slot
       continue;
     }
-    const uint32_t order = (k + teams - off) % teams;
+    const uint32_t order = (seat.k + teams - off) % teams;
     const Team tm{(int)(b - first), (int)T, tab.slot[0] + first, cx.hdr};
     if (t == 0) sh.gen = (uint32_t)L << kTeamGenBits;
     __syncthreads();
@@ -1289,7 +1282,7 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
         if (pos >= end) continue;
       }
       if (pos >= end) break;
-      const uint64_t si = own ? pos : team_slot;
+      const uint64_t si = own ? pos : seat.slot;
       if (!bounds_ok(cx.hdr, (si + 1) * need <= cx.scratch_bytes, kSiteFwdSlot)) continue;
       // (bulk copies need 16-byte addresses; a slot has room for the shift)
       float* slot = reinterpret_cast<float*>(align_up(reinterpret_cast<size_t>(cx.scratch + si * need), 16));

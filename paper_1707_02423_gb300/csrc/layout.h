@@ -344,6 +344,55 @@ CF_HD int team_level(int64_t cost, int64_t total, int n_cta) {
   return L;
 }
 
+// Where CTA b of the forward's team kernel works on a team level: the team's
+// size and number, its first CTA and its scratch slot (`in`: b is in a team).
+//   - A slot for every CTA (or for every pair, which then take their own): team
+//     k of level L has CTAs k T .. k T + T - 1, T = n_team >> L, and the slot of
+//     its first CTA.  Coarser teams with that first CTA hold all of its CTAs.
+//   - Fewer slots (shared): the two teams below a team lie inside it, side by
+//     side, and a team has the slot of the first of its finest teams.  So teams
+//     that use one slot on different levels lie inside one another, and as a
+//     team's last barrier keeps all of its CTAs until it is done (no barrier
+//     sits between levels), a CTA comes to a slot only when the slot's last team
+//     has left it.  (Slots dealt out in proportion to the first CTA don't do:
+//     152 CTAs make teams of 19 and of 9, which straddle one another, and CTA 18,
+//     free after team 0-18, would write to the slot that team 19-37 is using.)
+//     The finest level (team_finest) is the one whose teams all have a slot.
+struct TeamSeat {
+  uint32_t T, teams, k, first;
+  uint64_t slot;
+  bool in;
+};
+CF_HD int team_finest(uint32_t n_team, uint64_t nslots) {
+  int f = 0;
+  while (f + 1 < kTeamLevels - 1 && (n_team >> (f + 1)) > 0 && ((uint64_t)2 << f) <= nslots) ++f;
+  return f;
+}
+CF_HD TeamSeat team_seat(uint32_t b, int L, uint32_t n_team, uint32_t grid, bool shared, int finest) {
+  TeamSeat s{};
+  if (L == kTeamLevels - 1) {  // single CTAs
+    s = TeamSeat{1u, grid, b, b, b, b < grid};
+  } else if (shared) {
+    for (int l = 1; l <= L; ++l) {
+      const bool right = b >= s.first + (n_team >> l);
+      s.k = 2 * s.k + (right ? 1u : 0u);
+      if (right) s.first += n_team >> l;
+    }
+    s.T = n_team >> L;
+    s.teams = 1u << L;
+    s.slot = (uint64_t)s.k << (finest - L);
+    s.in = b >= s.first && b < s.first + s.T;
+  } else {
+    s.T = (n_team >> L) > 0 ? n_team >> L : 1u;
+    s.teams = n_team / s.T;
+    s.k = b / s.T;
+    s.first = s.k * s.T;
+    s.slot = s.first;
+    s.in = s.k < s.teams;
+  }
+  return s;
+}
+
 // Workspace header (first bytes of the workspace, zeroed at every call).
 struct WsHeader {
   int32_t status;       // first device-side error (cf_status code), 0 = none
