@@ -264,10 +264,12 @@ int device_sm_count() {
   return n;
 }
 
-// Scan the host pair list: validate and size the scratch slots of
-// global-class pairs (the class set is the same for the batched and the
-// per-pair forms).
-cf_status scan_pairs(const void* h_pack_a, const void* h_pack_b, const int32_t* h_pairs, int32_t P,
+// Scan the host pair list: validate it and size the scratch slots of the pairs
+// that fit no single CTA under a forward variant (its thread count: a long,
+// thin pair whose longer side is 513 to 1,024 fits a CTA of 1,024 threads
+// only, one column per thread).  Such pairs are the global class, or the
+// cluster class under a tune with clusters.
+cf_status scan_pairs(const void* h_pack_a, const void* h_pack_b, const int32_t* h_pairs, int32_t P, int variant,
                      int64_t* x_elems, int64_t* m_elems, size_t* slot_need, int64_t* n_global) {
   PackHeader ha, hb;
   cf_status s = read_header(h_pack_a, &ha, "h_pack_a");
@@ -285,8 +287,7 @@ cf_status scan_pairs(const void* h_pack_a, const void* h_pack_b, const int32_t* 
   const uint8_t* xdb = reinterpret_cast<const uint8_t*>(static_cast<const char*>(h_pack_b) + hb.off_xdeg);
   int64_t xs = 0, ms = 0, ng = 0;
   size_t need = 0;
-  // pairs that fit no single CTA: the global class, or the cluster class under a tune with clusters
-  const ClassCfg cc = fwd_class_cfg(0, kClassWarp, 0, 0);
+  const ClassCfg cc = fwd_class_cfg(variant, kClassWarp, 0, 0);
   for (int p = 0; p < P; ++p) {
     const int a = h_pairs[2 * p], b = h_pairs[2 * p + 1];
     if (a < 0 || a >= ha.n_cfgs || b < 0 || b >= hb.n_cfgs)
@@ -518,7 +519,7 @@ cf_status cf_pack_set_weights(void* d_pack, const void* h_pack, const float* d_w
 
 cf_status cf_out_sizes(const void* h_pack_a, const void* h_pack_b, const int32_t* h_pairs, int32_t P,
                        int64_t* x_elems, int64_t* match_elems) {
-  cf_status s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, x_elems, match_elems, nullptr, nullptr);
+  cf_status s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, 0, x_elems, match_elems, nullptr, nullptr);
   return s ? s : ok();
 }
 
@@ -531,7 +532,10 @@ cf_status cf_similarity_ws_size(const void* h_pack_a, const void* h_pack_b, cons
   }
   size_t need = 0;
   int64_t ng = 0, xs = 0;
-  cf_status s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, &xs, nullptr, &need, &ng);
+  // the plan's variant, whatever the form of the launch (without params: the default tune's)
+  const cf_params none{};
+  const int variant = call_tune(params ? params : &none, P).variant;
+  cf_status s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, variant, &xs, nullptr, &need, &ng);
   if (s) return s;
   // scratch slots for global-class pairs: one per concurrently working CTA
   // (the plain form spread over streams: one per stream)
@@ -639,7 +643,7 @@ cf_status cf_similarity_backward_ws_size(const void* h_pack_a, const void* h_pac
   if (s) return s;
   s = read_header(h_pack_b, &hb, "h_pack_b");
   if (s) return s;
-  s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, nullptr, nullptr, nullptr, nullptr);
+  s = scan_pairs(h_pack_a, h_pack_b, h_pairs, P, 0, nullptr, nullptr, nullptr, nullptr);
   if (s) return s;
   int variant = 0, cluster = 0;
   bwd_config(params, &variant, &cluster);

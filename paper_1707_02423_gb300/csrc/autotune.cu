@@ -78,9 +78,11 @@ cf_status tune_layout(const void* h_pack_a, const void* h_pack_b, const std::vec
   size_t ws = 0, ws3 = 0;
   cf_status s = cf_similarity_ws_size(h_pack_a, h_pack_b, sp.data(), S, params, &ws);
   if (s) return s;
-  cf_params p3 = *params;  // the candidates with deferred matching steps need room for the ranked lists
+  // the candidates with deferred matching steps need room for the ranked lists,
+  // those of 512 threads scratch slots for pairs that fit a CTA of more
+  cf_params p3 = *params;
   p3.flags = 0;
-  p3.tune = kFirstDeferTune;
+  p3.tune = kFirstDeferTune + 1;
   s = cf_similarity_ws_size(h_pack_a, h_pack_b, sp.data(), S, &p3, &ws3);
   if (s) return s;
   ws = std::max(ws, ws3);
