@@ -110,34 +110,6 @@ __device__ __forceinline__ Geo make_geo(const Ctx& cx, int p, const ClassCfg& cc
   return g;
 }
 
-// Same sum with both graphs' lists read from memory (global-class pairs).
-__device__ __forceinline__ float gather_g(const float* Y, int ld, const Geo& g, int i, int j) {
-  float s = 0.f;
-  const int c0 = __ldg(g.c_optr + j), c1 = __ldg(g.c_optr + j + 1);
-  for (int e = __ldg(g.r_optr + i), e1 = __ldg(g.r_optr + i + 1); e < e1; ++e) {
-    const CfAdj a = ldg_adj(g.r_oadj + e);
-    const float* row = Y + (size_t)a.nbr * ld;
-    float t = 0.f;
-    for (int f = c0; f < c1; ++f) {
-      const CfAdj b = ldg_adj(g.c_oadj + f);
-      t = fmaf(b.w, row[b.nbr], t);
-    }
-    s = fmaf(a.w, t, s);
-  }
-  const int d0 = __ldg(g.c_iptr + j), d1 = __ldg(g.c_iptr + j + 1);
-  for (int e = __ldg(g.r_iptr + i), e1 = __ldg(g.r_iptr + i + 1); e < e1; ++e) {
-    const CfAdj a = ldg_adj(g.r_iadj + e);
-    const float* row = Y + (size_t)a.nbr * ld;
-    float t = 0.f;
-    for (int f = d0; f < d1; ++f) {
-      const CfAdj b = ldg_adj(g.c_iadj + f);
-      t = fmaf(b.w, row[b.nbr], t);
-    }
-    s = fmaf(a.w, t, s);
-  }
-  return s;
-}
-
 // a5-a6: greedy matching by rounds of locally dominant entries, and the score.
 //
 // Sequential greedy takes the largest remaining entry under the strict order

@@ -272,6 +272,20 @@ __device__ __forceinline__ void mask_prefix(const uint32_t* m0, const uint32_t* 
   }
 }
 
+// Bit masks of the row graph's busy rows (more than two out- or in-neighbours),
+// twice.
+template <int NW>
+__device__ __forceinline__ void row_masks(const Geo& g, int n_row, int words, uint32_t* m0, uint32_t* mb, int lane,
+                                          int w) {
+  for (int wd = w; wd < words; wd += NW) {
+    const int i = 32 * wd + lane;
+    const bool busy = i < n_row && (__ldg(g.r_optr + i + 1) - __ldg(g.r_optr + i) > 2 ||
+                                    __ldg(g.r_iptr + i + 1) - __ldg(g.r_iptr + i) > 2);
+    const unsigned m = __ballot_sync(0xffffffffu, busy);
+    if (lane == 0) m0[wd] = mb[wd] = m;
+  }
+}
+
 // ---- the sweep: rows through a ring in shared memory -----------------------
 //
 // A slab's rows are swept in order, and every row they gather from comes
@@ -990,6 +1004,257 @@ __device__ __forceinline__ float team_iterate(const Team& tm, TeamSh& sh, const 
   return sk;
 }
 
+// The iterations of a pair whose graphs cannot be staged (rows too long for a
+// ring of them, about 3,800 columns and more): rows and column lists come from
+// memory, columns in natural order.  What bounds an iteration is the loads in
+// flight and the longest chain of list terms that one warp has, so
+//   - a slab's rows with at most two neighbours either way are swept by strips,
+//     32 columns and a run of rows a warp: the columns' first two neighbours
+//     stay in registers, the rows' records come from shared memory, and kFarRows
+//     rows' loads are issued before any is used;
+//   - the other rows (the STOP block has an in-edge from every early return) are
+//     shared out over the team's warps, 32 columns at a time;
+//   - an entry at a column with more than kFarList neighbours is the whole
+//     warp's, its lanes over the longer of the two lists.
+// One pair of 4,400 x 4,800 blocks, in-degree of the STOP block 129, K = 40: 14.8
+// ms; 152 pairs of 4,400-4,800: 2.59 s.  (Both lists read entry by entry, a lane
+// per column whatever its list, so that one warp had the STOP row and one lane
+// the entry at both STOP blocks: 542 ms and 77.5 s.  The busy rows shared out
+// but no strips, a column's lists read again at every row: 31 ms and 5.1 s.  One
+// CTA per pair: 3,400 ms and 4.7 s.)
+constexpr int kFarRows = 4;
+constexpr int kFarList = 16;
+constexpr int kFarBlock = 1024;        // rows whose records are staged at a time
+constexpr size_t kFarRecs = 1 << 16;   // their place, behind the list of the other rows
+
+// sum_e sum_f w_e w_f Y[u_e, v_f] over two lists: this lane's part.
+__device__ __forceinline__ float far_pair(const float* Y, uint32_t ld, const CfAdj* ra, int e0, int e1, const CfAdj* ca,
+                                          int f0, int f1, int lane) {
+  uint32_t sa = 1, sb = ld;  // strides: of the list over the lanes, of the other
+  if (e1 - e0 > f1 - f0) {
+    const CfAdj* a = ra;
+    ra = ca;
+    ca = a;
+    int k = e0;
+    e0 = f0;
+    f0 = k;
+    k = e1;
+    e1 = f1;
+    f1 = k;
+    sa = ld;
+    sb = 1;
+  }
+  float s = 0.f;
+  for (int f = f0 + lane; f < f1; f += 32) {
+    const CfAdj v = ldg_adj(ca + f);
+    const float* y = Y + sa * (uint32_t)v.nbr;
+    float z = 0.f;
+#pragma unroll 8
+    for (int e = e0; e < e1; ++e) {
+      const CfAdj u = ldg_adj(ra + e);
+      z = fmaf(u.w, y[sb * (uint32_t)u.nbr], z);
+    }
+    s = fmaf(v.w, z, s);
+  }
+  return s;
+}
+
+// The same at this lane's column, whose list is short.
+__device__ __forceinline__ float far_lane(const float* Y, uint32_t ld, const CfAdj* ra, int e0, int e1, const CfAdj* ca,
+                                          int f0, int f1) {
+  float s = 0.f;
+  for (int f = f0; f < f1; ++f) {
+    const CfAdj v = ldg_adj(ca + f);
+    float z = 0.f;
+#pragma unroll 8
+    for (int e = e0; e < e1; ++e) {
+      const CfAdj u = ldg_adj(ra + e);
+      z = fmaf(u.w, Y[(uint32_t)u.nbr * ld + (uint32_t)v.nbr], z);
+    }
+    s = fmaf(v.w, z, s);
+  }
+  return s;
+}
+
+// A lane's column: its lists' ranges and first two neighbours (a missing one
+// has weight 0).
+struct FarCol {
+  int c0, c1, d0, d1;
+  uint32_t vo0, vo1, vi0, vi1;
+  float wo0, wo1, wi0, wi1;
+};
+__device__ __forceinline__ FarCol far_col(const Geo& g, int j, int n_col) {
+  FarCol c{};
+  if (j < n_col) {
+    c.c0 = __ldg(g.c_optr + j);
+    c.c1 = __ldg(g.c_optr + j + 1);
+    c.d0 = __ldg(g.c_iptr + j);
+    c.d1 = __ldg(g.c_iptr + j + 1);
+    const CfAdj z{0, 0.f};
+    const CfAdj a0 = c.c1 > c.c0 ? ldg_adj(g.c_oadj + c.c0) : z, a1 = c.c1 > c.c0 + 1 ? ldg_adj(g.c_oadj + c.c0 + 1) : z;
+    const CfAdj b0 = c.d1 > c.d0 ? ldg_adj(g.c_iadj + c.d0) : z, b1 = c.d1 > c.d0 + 1 ? ldg_adj(g.c_iadj + c.d0 + 1) : z;
+    c.vo0 = (uint32_t)a0.nbr;
+    c.vo1 = (uint32_t)a1.nbr;
+    c.vi0 = (uint32_t)b0.nbr;
+    c.vi1 = (uint32_t)b1.nbr;
+    c.wo0 = a0.w;
+    c.wo1 = a1.w;
+    c.wi0 = b0.w;
+    c.wi1 = b1.w;
+  }
+  return c;
+}
+
+// Rows i0 + r .. of the staged records (r + kFarRows > r1: the last ones are
+// left out) at the lanes' columns.  A record: {4 out 0, out 1, in 0, in 1: ld
+// times the row}, their weights; x = ~0: not one of these rows.
+__device__ __forceinline__ float far_rows(const Geo& g, const float* Y, float* nxt, const float* eb, uint32_t ld, int i0,
+                                          const int4* rec, int r, int r1, const FarCol& c, bool big, int j, int n_col,
+                                          float ca, float cbi, int lane) {
+  int4 A[kFarRows], W[kFarRows];
+  float s0[kFarRows], s1[kFarRows], t0[kFarRows], t1[kFarRows], e[kFarRows], z[kFarRows];
+#pragma unroll
+  for (int u = 0; u < kFarRows; ++u) {
+    const int q = min(r + u, r1 - 1);
+    A[u] = rec[2 * q];
+    W[u] = rec[2 * q + 1];
+    const uint32_t o = A[u].x == -1 ? 0u : (uint32_t)A[u].x;
+    s0[u] = Y[o + c.vo0];
+    s1[u] = Y[(uint32_t)A[u].z + c.vi0];
+    t0[u] = Y[o + c.vo1];
+    t1[u] = Y[(uint32_t)A[u].z + c.vi1];
+    e[u] = j < n_col ? eb[(uint32_t)(i0 + q) * ld + (uint32_t)j] : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < kFarRows; ++u) {
+    z[u] = __int_as_float(W[u].x) * fmaf(c.wo1, t0[u], c.wo0 * s0[u]) +
+           __int_as_float(W[u].z) * fmaf(c.wi1, t1[u], c.wi0 * s1[u]);
+    if ((W[u].y | W[u].w) != 0) {
+      const float* y1 = Y + (uint32_t)A[u].y;
+      const float* y2 = Y + (uint32_t)A[u].w;
+      z[u] += __int_as_float(W[u].y) * fmaf(c.wo1, y1[c.vo1], c.wo0 * y1[c.vo0]) +
+              __int_as_float(W[u].w) * fmaf(c.wi1, y2[c.vi1], c.wi0 * y2[c.vi0]);
+    }
+  }
+  // further neighbours: the lane's, or over the warp
+  auto terms = [&](const CfAdj v, bool in, float (&s)[kFarRows]) {
+#pragma unroll
+    for (int u = 0; u < kFarRows; ++u) {
+      const uint32_t a = in ? (uint32_t)A[u].z : A[u].x == -1 ? 0u : (uint32_t)A[u].x, b = (uint32_t)(in ? A[u].w : A[u].y);
+      const float wa = __int_as_float(in ? W[u].z : W[u].x), wb = __int_as_float(in ? W[u].w : W[u].y);
+      float y = wa * Y[a + (uint32_t)v.nbr];
+      if (wb != 0.f) y = fmaf(wb, Y[b + (uint32_t)v.nbr], y);
+      s[u] = fmaf(v.w, y, s[u]);
+    }
+  };
+  if (!big) {
+    for (int f = c.c0 + 2; f < c.c1; ++f) terms(ldg_adj(g.c_oadj + f), false, z);
+    for (int f = c.d0 + 2; f < c.d1; ++f) terms(ldg_adj(g.c_iadj + f), true, z);
+  }
+  for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+    const int l = __ffs(m) - 1;
+    const int f0 = __shfl_sync(0xffffffffu, c.c0, l) + 2, f1 = __shfl_sync(0xffffffffu, c.c1, l);
+    const int h0 = __shfl_sync(0xffffffffu, c.d0, l) + 2, h1 = __shfl_sync(0xffffffffu, c.d1, l);
+    float s[kFarRows] = {};
+    for (int f = f0 + lane; f < f1; f += 32) terms(ldg_adj(g.c_oadj + f), false, s);
+    for (int f = h0 + lane; f < h1; f += 32) terms(ldg_adj(g.c_iadj + f), true, s);
+#pragma unroll
+    for (int u = 0; u < kFarRows; ++u) {
+      const float v = warp_sum(s[u]);
+      if (lane == l) z[u] += v;
+    }
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int u = 0; u < kFarRows; ++u)
+    if (r + u < r1 && A[u].x != -1 && j < n_col) {
+      const float y = fmaf(ca, z[u], cbi * e[u]);
+      nxt[(uint32_t)(i0 + r + u) * ld + (uint32_t)j] = y;
+      ss = fmaf(y, y, ss);
+    }
+  return ss;
+}
+
+// region: the rows of the row graph with more than two neighbours (nbr of
+// them), then room for the records; i0, i1: this CTA's slab.  Returns s_K.
+template <int NT>
+__device__ __noinline__ float team_far(const Team& tm, TeamSh& sh, const TeamIter& it, const Geo& g, uint32_t ld, int i0,
+                                       int i1, unsigned char* region, int nbr) {
+  constexpr int NW = NT / 32;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, n_col = g.nb;
+  const int nch = ceil_div(n_col, 32);
+  const uint16_t* rows = reinterpret_cast<const uint16_t*>(region);
+  int4* rec = reinterpret_cast<int4*>(region + kFarRecs);
+  float sk = it.s0;
+  for (int k = 0; k < it.K; ++k) {
+    const float* Y = iter_from(it, k);
+    float* nxt = iter_to(it, k);
+    const float ca = 0.5f * it.alpha * sk;
+    float ss = 0.f;
+    // the longest first
+    for (int64_t q = (int64_t)w * tm.T + tm.c; q < (int64_t)nbr * nch; q += NW * tm.T) {
+      const int b = (int)(q / nch), j = 32 * (int)(q - (int64_t)b * nch) + lane, i = rows[b];
+      const int o0 = __ldg(g.r_optr + i), o1 = __ldg(g.r_optr + i + 1);
+      const int q0 = __ldg(g.r_iptr + i), q1 = __ldg(g.r_iptr + i + 1);
+      int c0 = 0, c1 = 0, d0 = 0, d1 = 0;
+      if (j < n_col) {
+        c0 = __ldg(g.c_optr + j);
+        c1 = __ldg(g.c_optr + j + 1);
+        d0 = __ldg(g.c_iptr + j);
+        d1 = __ldg(g.c_iptr + j + 1);
+      }
+      const bool big = c1 - c0 > kFarList || d1 - d0 > kFarList;
+      float z = 0.f;
+      if (!big)
+        z = far_lane(Y, ld, g.r_oadj, o0, o1, g.c_oadj, c0, c1) + far_lane(Y, ld, g.r_iadj, q0, q1, g.c_iadj, d0, d1);
+      for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        const int f0 = __shfl_sync(0xffffffffu, c0, l), f1 = __shfl_sync(0xffffffffu, c1, l);
+        const int h0 = __shfl_sync(0xffffffffu, d0, l), h1 = __shfl_sync(0xffffffffu, d1, l);
+        const float v = warp_sum(far_pair(Y, ld, g.r_oadj, o0, o1, g.c_oadj, f0, f1, lane) +
+                                 far_pair(Y, ld, g.r_iadj, q0, q1, g.c_iadj, h0, h1, lane));
+        if (lane == l) z = v;
+      }
+      if (j < n_col) {
+        const uint32_t at = (uint32_t)i * ld + (uint32_t)j;
+        const float y = fmaf(ca, z, it.cbi * it.eb[at]);
+        nxt[at] = y;
+        ss = fmaf(y, y, ss);
+      }
+    }
+    for (int b0 = i0; b0 < i1; b0 += kFarBlock) {
+      const int nr = min(kFarBlock, i1 - b0);
+      if (k == 0 || i1 - i0 > kFarBlock) {
+        __syncthreads();
+        for (int r = t; r < nr; r += NT) {
+          const int o0 = __ldg(g.r_optr + b0 + r), o1 = __ldg(g.r_optr + b0 + r + 1);
+          const int q0 = __ldg(g.r_iptr + b0 + r), q1 = __ldg(g.r_iptr + b0 + r + 1);
+          const bool in = o1 - o0 <= 2 && q1 - q0 <= 2;
+          const CfAdj z{0, 0.f};
+          const CfAdj a0 = in && o1 > o0 ? ldg_adj(g.r_oadj + o0) : z, a1 = in && o1 > o0 + 1 ? ldg_adj(g.r_oadj + o0 + 1) : z;
+          const CfAdj d0 = in && q1 > q0 ? ldg_adj(g.r_iadj + q0) : z, d1 = in && q1 > q0 + 1 ? ldg_adj(g.r_iadj + q0 + 1) : z;
+          rec[2 * r] = make_int4(in ? (int)((uint32_t)a0.nbr * ld) : -1, (int)((uint32_t)a1.nbr * ld),
+                                 (int)((uint32_t)d0.nbr * ld), (int)((uint32_t)d1.nbr * ld));
+          rec[2 * r + 1] = make_int4(__float_as_int(a0.w), __float_as_int(a1.w), __float_as_int(d0.w), __float_as_int(d1.w));
+        }
+        __syncthreads();
+      }
+      // strips: every warp some, whatever the matrix's shape
+      const int runs = min(ceil_div(nr, kFarRows), ceil_div(4 * NW, nch)), len = ceil_div(nr, runs);
+      for (int q = w; q < nch * runs; q += NW) {
+        const int h = q % nch, r0 = q / nch * len, r1 = min(nr, r0 + len), j = 32 * h + lane;
+        const FarCol c = far_col(g, j, n_col);
+        const bool big = c.c1 - c.c0 > kFarList || c.d1 - c.d0 > kFarList;
+        for (int r = r0; r < r1; r += kFarRows)
+          ss += far_rows(g, Y, nxt, it.eb, ld, b0, rec, r, r1, c, big, j, n_col, ca, it.cbi, lane);
+      }
+    }
+    const float yy = team_sum(tm, sh, ss);
+    sk = it.norm_mode == 0 ? 1.0f / sqrtf(yy) : 1.f;
+  }
+  return sk;
+}
+
 // ---------------------------------------------------------------------------
 // The greedy matching of a team's pair, in phases.  X_K is close to rank one,
 // so the sequential greedy takes its entries nearly one at a time, and rounds
@@ -1634,13 +1899,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
     }
     __syncthreads();
     // the row graph's busy rows, in index order
-    for (int wd = w; wd < words; wd += NW) {
-      const int i = 32 * wd + lane;
-      const bool busy = i < n_row && (__ldg(g.r_optr + i + 1) - __ldg(g.r_optr + i) > 2 ||
-                                      __ldg(g.r_iptr + i + 1) - __ldg(g.r_iptr + i) > 2);
-      const unsigned m = __ballot_sync(0xffffffffu, busy);
-      if (lane == 0) m0[wd] = mb[wd] = m;
-    }
+    row_masks<NW>(g, n_row, words, m0, mb, lane, w);
     __syncthreads();
     if (w == 0) mask_prefix(m0, mb, p0, pb, words, lane, &sh.nbs, &sh.nbs);
     __syncthreads();
@@ -1716,6 +1975,17 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
     if (w == NC + kBusyWarps) team_schedule(sh.st, rec, last, use, what, lane);
     if (w == NC) busy_lanes(sh.st, bran, blane, lane);
   }
+  if (!staged) {  // the rows with more than two neighbours, in index order
+    uint16_t* rows = reinterpret_cast<uint16_t*>(region);
+    row_masks<NW>(g, n_row, words, m0, mb, lane, w);
+    __syncthreads();
+    if (w == 0) mask_prefix(m0, mb, p0, pb, words, lane, &sh.nbs, &sh.nbs);
+    __syncthreads();
+    for (int i = t; i < n_row; i += NT) {
+      const uint32_t m = m0[i >> 5], bit = 1u << (i & 31);
+      if (m & bit) rows[p0[i >> 5] + __popc(m & (bit - 1u))] = (uint16_t)i;
+    }
+  }
   const uint16_t* cnat = reinterpret_cast<const uint16_t*>(region);
   for (int i = i0 + t; i < i1; i += NT) rn[i] = attr_norm(g.r_attr + (size_t)i * cx.Fp, cx.om, cx.Fp);
   __syncthreads();
@@ -1777,22 +2047,9 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
   if (staged) {
     const TeamIter it{eb, b0, b1, cx.alpha, inv, cbi, cx.K, cx.norm_mode};
     sk = team_iterate<NT>(tm, sh, it, CH);
-  } else {  // graphs too large to stage: both graphs' lists from memory, natural order
-    for (int k = 0; k < cx.K; ++k) {
-      const float* cur = k == 0 ? eb : ((cx.K - k) & 1) ? b1 : b0;
-      float* nxt = ((cx.K - 1 - k) & 1) ? b1 : b0;
-      const float ca = 0.5f * cx.alpha * sk;
-      ss = 0.f;
-      for (int i = i0 + w; i < i1; i += NW)
-        for (int j = lane; j < n_col; j += 32) {
-          const size_t q = (size_t)i * ld + j;
-          const float y = fmaf(ca, gather_g(cur, (int)ld, g, i, j), cbi * eb[q]);
-          nxt[q] = y;
-          ss = fmaf(y, y, ss);
-        }
-      const float yy = team_sum(tm, sh, ss);
-      sk = cx.norm_mode == 0 ? 1.0f / sqrtf(yy) : 1.f;
-    }
+  } else {
+    sk = team_far<NT>(tm, sh, TeamIter{eb, b0, b1, cx.alpha, inv, cbi, cx.K, cx.norm_mode}, g, ld, i0, i1,
+                      region, nbr);
   }
   // X_K in the caller's column order (rows of n_col): to the output, and for
   // the matching into b1 (the matching's lists then take E and b0)
