@@ -193,7 +193,8 @@ CF_HD Shape classify(int na, int nb, int ea, int eb, const ClassCfg& c, int xa =
     const size_t Z = group_region(cls, c);
     int R0 = 0, M0 = 0, R1 = 0, M1 = 0;
     const bool f0 = fits(na, nb, ea, eb, G, Z, &R0, &M0, c.bwd);
-    const bool f1 = fits(nb, na, eb, ea, G, Z, &R1, &M1, c.bwd);
+    // (the matching alone keeps the caller's orientation)
+    const bool f1 = c.bwd != 2 && fits(nb, na, eb, ea, G, Z, &R1, &M1, c.bwd);
     if (f0 || f1) {
       const bool tr = !f0 || (f1 && prefer_tr(M0, M1, xa, xb));
       s.cls = cls;
