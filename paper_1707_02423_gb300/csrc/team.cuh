@@ -1732,6 +1732,7 @@ __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const 
     const float sc = greedy<int32_t>(cta, X, n_col, n_row, n_col, 0, ms, ms + n_row, ms + n_row + n_col, mo, cx.hdr,
                                      g.p);
     if (cx.scores && t == 0) cx.scores[g.p] = sc;
+    __syncthreads();  // team_sum takes redw, which greedy's last sum was read from
   }
   team_sum(tm, sh, 0.f);
 }
