@@ -1481,27 +1481,39 @@ __device__ __forceinline__ int team_steps(TeamSh& sh, int nl, int left, const ui
   return made;
 }
 
-// Shared memory of a phase: the column flags, the listed rows and their
-// lengths, then the larger of the warps' candidates (with the bins) and the
-// lists with their column numbers.
+// Shared memory of a phase: the listed rows and their lengths, then the larger
+// of the column flags with the warps' candidates (or the bins) and, where those
+// are no longer read, the lists with their column numbers.
 constexpr int kIds = 680;  // columns a phase numbers; a list ends before its first column without a number
-__device__ __forceinline__ size_t greedy_team_bytes(int n_col, int NT) {
-  const size_t a = sizeof(uint2) * kCand * (NT / 32);
+constexpr size_t kListBytes = kTop * (8 * (size_t)kLen + 4);  // scratch: the lists, their lengths
+__device__ __forceinline__ size_t greedy_team_bytes(int n_col, int NT, bool wide) {
+  const size_t a = align_up((size_t)n_col, 16) + sizeof(uint2) * kCand * (NT / 32);
   const size_t b = (4 * (size_t)kKeyPitch + 2 * (size_t)kColPitch) * kLen + kIds * (size_t)kTop + 2 * kIds +
-                   align_up(2 * (size_t)n_col, 16);
-  return align_up((size_t)n_col, 16) + 2 * kTop + 4 * kTop + (a > b ? a : b);
+                   (wide ? 0 : align_up(2 * (size_t)n_col, 16));
+  return 2 * kTop + 4 * kTop + (a > b ? a : b);
 }
-// Whether greedy_team can take the pair (the caller falls back to greedy()).
-__device__ __forceinline__ bool greedy_team_fits(int n_row, int n_col, int NT, int region_bytes) {
-  return NT >= kTop && n_row <= kTeamRowsPer * NT && greedy_team_bytes(n_col, NT) <= (size_t)region_bytes &&
-         (size_t)n_row * n_col >= (2 * kLen + 1) * (size_t)kTop / 2;
+// The forms of greedy_team: rows in registers and the columns' numbers in
+// shared memory; beyond (5,120 rows, 10,616 columns: wide) the rows' best
+// values are read where they are needed and the columns' numbers lie behind the
+// lists.  Neither takes a matrix that is smaller than the lists' scratch: for
+// the few thousand entries of a thin one greedy() is enough.
+enum GreedyForm { kGreedySmall, kGreedyTeam, kGreedyWide };
+__device__ __forceinline__ GreedyForm greedy_form(int n_row, int n_col, int NT, int region_bytes) {
+  const bool wide = n_row > kTeamRowsPer * NT || greedy_team_bytes(n_col, NT, false) > (size_t)region_bytes;
+  if (NT < kTop || greedy_team_bytes(n_col, NT, wide) > (size_t)region_bytes ||
+      8 * (size_t)n_row * n_col < kListBytes + (wide ? 2 * (size_t)n_col : 0))
+    return kGreedySmall;
+  return wide ? kGreedyWide : kGreedyTeam;
 }
 
 // X: the pair's X_K (or a caller's matrix), row-major n_row x n_col, complete
-// and visible to the team.  lists: kTop x (2 kLen + 1) words of scratch; ms:
-// n_row ints (row matches), then n_col bytes (column flags); best: n_row
-// ints.  Ends with a team barrier.  Returns the score on every thread.
-template <int NT>
+// and visible to the team.  lists: scratch of 8 n_row n_col bytes; ms: n_row
+// ints (row matches), then n_col bytes (column flags); best: n_row ints.  Ends
+// with a team barrier.  Returns the score on every thread.
+// (5,200 x 5,200 given, near rank one: 11.5 ms in the wide form, 5,000 x 5,200 8.9
+// ms in the other; one CTA with greedy(), the team waiting, 7.6 s.  152 such pairs:
+// 1.52 s, against 12.4 s with a CTA per pair.)
+template <int NT, bool kWide>
 __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const float* X, int n_row, int n_col,
                                           uint2* lists, int32_t* ms, uint32_t* best, unsigned char* region,
                                           int32_t* mo, int pidx) {
@@ -1511,11 +1523,12 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
   int32_t* mrow = ms;
   unsigned char* gdead = reinterpret_cast<unsigned char*>(ms + n_row);
   int* glen = reinterpret_cast<int*>(lists + kTop * kLen);
-  unsigned char* dead = region;
-  uint16_t* sel = reinterpret_cast<uint16_t*>(region + align_up((size_t)n_col, 16));
+  uint16_t* sel = reinterpret_cast<uint16_t*>(region);
   int* len = reinterpret_cast<int*>(sel + kTop);
-  unsigned char* rest = reinterpret_cast<unsigned char*>(len + kTop);
-  const int K = min(kLen, n_col);
+  unsigned char* dead = reinterpret_cast<unsigned char*>(len + kTop);
+  unsigned char* rest = dead + align_up((size_t)n_col, 16);
+  int* pre = kWide ? reinterpret_cast<int*>(rest) + kBins : &sh.pre[0][0];  // [rows' block][warp]
+  const int K = min(kLen, n_col), M = kWide ? ceil_div(n_row, NT) : kTeamRowsPer;
   for (int i = i0 + t; i < i1; i += NT) mrow[i] = -1;
   if (tm.c == 0)
     for (int j = t; j < n_col; j += NT) gdead[j] = 0;
@@ -1549,13 +1562,22 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     // the listed rows (every CTA finds the same ones): all rows down to a bin
     // of best values, at most kTop of them
     uint32_t v[kTeamRowsPer];
+    if constexpr (!kWide) {
+#pragma unroll
+      for (int m = 0; m < kTeamRowsPer; ++m) v[m] = t + NT * m < n_row ? best[t + NT * m] : 0u;
+    }
+    auto value = [&](int m) -> uint32_t {
+      if constexpr (kWide)
+        return t + NT * m < n_row ? best[t + NT * m] : 0u;
+      else
+        return v[m];
+    };
     uint32_t vmax = 0, vmin = 0xffffffffu;
 #pragma unroll
-    for (int m = 0; m < kTeamRowsPer; ++m) {
-      const int i = t + NT * m;
-      v[m] = i < n_row ? best[i] : 0u;
-      vmax = max(vmax, v[m]);
-      if (v[m]) vmin = min(vmin, v[m]);
+    for (int m = 0; m < M; ++m) {
+      const uint32_t k = value(m);
+      vmax = max(vmax, k);
+      if (k) vmin = min(vmin, k);
     }
     const uint64_t mm = block_max2<NW>(sh, vmax, ~vmin, lane, w);
     vmax = (uint32_t)(mm >> 32);
@@ -1563,8 +1585,10 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     vmin = ~(uint32_t)mm;
     const int shift = max(0, 32 - __clz(vmax - vmin) - 8);
 #pragma unroll
-    for (int m = 0; m < kTeamRowsPer; ++m)
-      if (v[m]) atomicAdd(&bins[(vmax - v[m]) >> shift], 1);
+    for (int m = 0; m < M; ++m) {
+      const uint32_t k = value(m);
+      if (k) atomicAdd(&bins[(vmax - k) >> shift], 1);
+    }
     __syncthreads();
     if (w == 0) {  // the last bin that keeps the count within kTop
       int run = 0, last = -1;
@@ -1587,41 +1611,41 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     const int bin = sh.bin;
     // (the first bin alone may hold more than kTop rows, many of equal value:
     // then the largest value's rows by index, up to kTop)
-    bool in[kTeamRowsPer];
+    auto listed = [&](uint32_t k) { return k != 0u && (bin >= 0 ? (int)((vmax - k) >> shift) <= bin : k == vmax); };
     uint64_t below = 0;  // the best row that is not listed
-    int cnt[kTeamRowsPer];
 #pragma unroll
-    for (int m = 0; m < kTeamRowsPer; ++m) {
-      in[m] = v[m] != 0u && (bin >= 0 ? (int)((vmax - v[m]) >> shift) <= bin : v[m] == vmax);
-      const unsigned b = __ballot_sync(0xffffffffu, in[m]);
-      cnt[m] = __popc(b & ((1u << lane) - 1u));
-      if (lane == 0) sh.pre[m][w] = __popc(b);
+    for (int m = 0; m < M; ++m) {
+      const unsigned b = __ballot_sync(0xffffffffu, listed(value(m)));
+      if (lane == 0) pre[32 * m + w] = __popc(b);
     }
     __syncthreads();
     if (w == 0) {  // exclusive prefix over (m, warp)
       int run = 0;
       for (int e0 = 0; e0 < NW * ceil_div(n_row, NT); e0 += 32) {
         const int m = (e0 + lane) / NW, q = (e0 + lane) % NW;
-        const int c = m < kTeamRowsPer ? sh.pre[m][q] : 0;
+        const int c = m < M ? pre[32 * m + q] : 0;
         int inc = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int u = __shfl_up_sync(0xffffffffu, inc, o);
           if (lane >= o) inc += u;
         }
-        if (m < kTeamRowsPer) sh.pre[m][q] = run + inc - c;
+        if (m < M) pre[32 * m + q] = run + inc - c;
         run += __shfl_sync(0xffffffffu, inc, 31);
       }
       if (lane == 0) sh.nl = min(run, kTop);
     }
     __syncthreads();
 #pragma unroll
-    for (int m = 0; m < kTeamRowsPer; ++m) {
-      const int i = t + NT * m, at = in[m] ? sh.pre[m][w] + cnt[m] : kTop;
+    for (int m = 0; m < M; ++m) {
+      const uint32_t k = value(m);
+      const bool in = listed(k);
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      const int i = t + NT * m, at = in ? pre[32 * m + w] + __popc(b & ((1u << lane) - 1u)) : kTop;
       if (at < kTop) {
         sel[at] = (uint16_t)i;
-      } else if (v[m]) {
-        const uint64_t q = ((uint64_t)v[m] << 16) | (uint32_t)(0xffff - i);
+      } else if (k) {
+        const uint64_t q = ((uint64_t)k << 16) | (uint32_t)(0xffff - i);
         below = q > below ? q : below;
       }
     }
@@ -1635,11 +1659,12 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     team_sum(tm, sh, 0.f);
     int made = 0;
     if (tm.c == 0) {
-      uint32_t* key = reinterpret_cast<uint32_t*>(rest);
+      uint32_t* key = reinterpret_cast<uint32_t*>(dead);  // the flags and candidates are done with
       uint16_t* col = reinterpret_cast<uint16_t*>(key + kKeyPitch * kLen);
       unsigned char* inv = reinterpret_cast<unsigned char*>(col + kColPitch * kLen);
       uint16_t* idcol = reinterpret_cast<uint16_t*>(inv + kIds * kTop);
-      unsigned short* id = reinterpret_cast<unsigned short*>(idcol + kIds);  // column -> number
+      unsigned short* id = kWide ? reinterpret_cast<unsigned short*>(lists) + kListBytes / 2
+                                 : reinterpret_cast<unsigned short*>(idcol + kIds);  // column -> number
       for (int s = t; s < nl; s += NT) len[s] = glen[s];
       for (int q = t; q < kIds * kTop / 16; q += NT)
         reinterpret_cast<uint4*>(inv)[q] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
@@ -1720,9 +1745,13 @@ __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const 
   float* rn = slot + 3 * (size_t)n_row * team_ld(n_col);
   int32_t* ms = reinterpret_cast<int32_t*>(rn + n_row + n_col);
   int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
-  if (greedy_team_fits(n_row, n_col, NT, region_bytes)) {
-    const float sc = greedy_team<NT>(tm, sh, X, n_row, n_col, reinterpret_cast<uint2*>(lists), ms,
-                                     reinterpret_cast<uint32_t*>(rn), region, mo, g.p);
+  const GreedyForm form = greedy_form(n_row, n_col, NT, region_bytes);
+  if (form != kGreedySmall) {
+    uint2* ls = reinterpret_cast<uint2*>(lists);
+    uint32_t* best = reinterpret_cast<uint32_t*>(rn);
+    const float sc = form == kGreedyWide
+                         ? greedy_team<NT, true>(tm, sh, X, n_row, n_col, ls, ms, best, region, mo, g.p)
+                         : greedy_team<NT, false>(tm, sh, X, n_row, n_col, ls, ms, best, region, mo, g.p);
     if (cx.scores && tm.c == 0 && t == 0) cx.scores[g.p] = sc;
     return;
   }
