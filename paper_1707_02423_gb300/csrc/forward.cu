@@ -110,6 +110,16 @@ __device__ __forceinline__ Geo make_geo(const Ctx& cx, int p, const ClassCfg& cc
   return g;
 }
 
+// Terms of an iteration of pair p, as the plan counts them.
+__device__ __forceinline__ int64_t pair_cost(const Ctx& cx, int p) {
+  const int pa = __ldg(cx.pairs + 2 * p), pb = __ldg(cx.pairs + 2 * p + 1);
+  const int64_t na = __ldg(cx.A.node_off + pa + 1) - __ldg(cx.A.node_off + pa);
+  const int64_t nb = __ldg(cx.B.node_off + pb + 1) - __ldg(cx.B.node_off + pb);
+  const int64_t ea = __ldg(cx.A.edge_off + pa + 1) - __ldg(cx.A.edge_off + pa);
+  const int64_t eb = __ldg(cx.B.edge_off + pb + 1) - __ldg(cx.B.edge_off + pb);
+  return na * nb + 2 * ea * eb;
+}
+
 // a5-a6: greedy matching by rounds of locally dominant entries, and the score.
 //
 // Sequential greedy takes the largest remaining entry under the strict order
@@ -1129,6 +1139,7 @@ __global__ void __launch_bounds__(NT, 1) fwd_batched_kernel(CallArgs a, int per_
             if (t == 0) {
               s_team.gen = 0;
               s_team.fail = 0;
+              s_team.wait = team_wait_ns(pair_cost(cx, per_pair));
             }
             __syncthreads();
             run_pair_t<NT>(cx, g, Team{0, 1, nullptr, cx.hdr}, s_team, pslot, smem, cc.z_cta);
@@ -1179,6 +1190,7 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
     sh.gen = 0;
     sh.fail = 0;
   }
+  if (t == 32) sh.wait = team_wait_ns(2 * pair_cost(cx, (int)cx.queue[0]));  // (in order to within a factor of two)
   const uint32_t b = blockIdx.x, grid = gridDim.x;
   const uint64_t need = cx.hdr->slot_need;
   const uint64_t nslots = need ? cx.scratch_bytes / need : 0;
@@ -1222,6 +1234,7 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
       fence_gpu();
     }
     __syncthreads();
+    if (sh.fail) return;
   }
   uint32_t beg = 0, cum = 0;
   for (int L = coop ? 0 : kTeamLevels - 1; L <= finest; ++L) {
@@ -1263,9 +1276,11 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
         match_pair_t<kTeamNT>(cx, g, tm, sh, slot, cx.X_in + cx.x_off[g.p], slot, smem, kTeamSmem);
       else
         run_pair_t<kTeamNT>(cx, g, tm, sh, slot, smem, kTeamSmem);
+      if (sh.fail) return;
       used = true;
     }
     if (used) team_leave(tm, sh);
+    if (sh.fail) return;
     beg = end;
   }
 }

@@ -394,6 +394,26 @@ CF_HD TeamSeat team_seat(uint32_t b, int L, uint32_t n_team, uint32_t grid, bool
   return s;
 }
 
+// A wait for a CTA of the team: over once that CTA has shown no progress (its
+// barrier word is the same) for `limit` ns.  Before a team's first barrier on a
+// level a CTA may still be at work on pairs of the level before, for as long as
+// those take, but it passes barriers all the while.
+struct TeamWait {
+  uint64_t since, seen;
+};
+CF_HD bool team_wait_over(TeamWait& w, uint64_t now, uint64_t word, uint64_t limit) {
+  if (word != w.seen) {
+    w.seen = word;
+    w.since = now;
+  }
+  return now - w.since > limit;
+}
+// What lies between two barriers is at most an iteration of a pair or a phase
+// of its matching, shared out evenly: fewer than four terms per ns and team
+// even on one CTA.  cost: of the costliest pair (the plan's).
+constexpr uint64_t kTeamWaitNs = 20ull * 1000 * 1000 * 1000;
+CF_HD uint64_t team_wait_ns(int64_t cost) { return kTeamWaitNs + 4 * (uint64_t)cost; }
+
 // Workspace header (first bytes of the workspace, zeroed at every call).
 struct WsHeader {
   int32_t status;       // first device-side error (cf_status code), 0 = none

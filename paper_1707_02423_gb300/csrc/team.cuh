@@ -102,7 +102,8 @@ struct TeamSh {
   int redi[64];
   float tot;
   uint32_t gen;    // level << kTeamGenBits | barriers passed in it
-  int fail;        // a wait ran out: no further waits
+  int fail;        // a wait ran out: the CTA waits no more and leaves the kernel
+  uint64_t wait;   // longest wait (team_wait_ns)
   int n0, nb, tb, tbp;           // columns: first kind, busy, list entries of the busy ones
   int nbs, nbr, tr, trp;         // busy rows, their list entries
   uint64_t red[32];      // per-warp maxima
@@ -135,11 +136,11 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// Longest wait for another CTA of the team (it only waits for work that is
-// itself bounded: the CTAs are co-resident, the kernel being launched
-// cooperatively).  A wait that runs out sets CF_ERR_TIMEOUT and the CTA goes
-// on without waiting, so the kernel ends.
-constexpr uint64_t kTeamWaitNs = 20ull * 1000 * 1000 * 1000;
+// Waits are bounded: for another CTA of the team (the CTAs are co-resident, the
+// kernel being launched cooperatively) by team_wait_over, within the CTA by the
+// same time.  One that runs out sets CF_ERR_TIMEOUT; the CTA then takes no
+// further part, as what it read may be unfinished: it leaves the pair without
+// using any of it as an index, and the kernel.
 
 // Sum of v over every thread of the team, the same bits on every thread, and
 // a barrier: what any thread of the team wrote before is visible to all of
@@ -165,11 +166,11 @@ __device__ __forceinline__ float team_sum(const Team& tm, TeamSh& sh, float v) {
       for (int k = lane; k < tm.T; k += 32) {
         uint64_t got = ld_relaxed_u64(s + k);
         if ((uint32_t)(got >> 32) != want && !sh.fail) {
-          const uint64_t t0 = global_ns();
+          TeamWait wait{global_ns(), got};
           for (uint32_t n = 0;; ++n) {
             got = ld_relaxed_u64(s + k);
             if ((uint32_t)(got >> 32) == want) break;
-            if ((n & 255u) == 255u && global_ns() - t0 > kTeamWaitNs) {
+            if ((n & 255u) == 255u && team_wait_over(wait, global_ns(), got, sh.wait)) {
               set_status(tm.hdr, 5 /* CF_ERR_TIMEOUT */, tm.c);
               sh.fail = 1;
               break;
@@ -230,13 +231,17 @@ __device__ __forceinline__ void team_leave(const Team& tm, TeamSh& sh) {
       fence_gpu();
       st_release_u64(s + tm.c, (uint64_t)want << 32);
     }
-    const uint64_t t0 = global_ns();
-    for (int k = lane; k < tm.T; k += 32)
-      while ((uint32_t)(ld_relaxed_u64(s + k) >> 32) < want && !*reinterpret_cast<volatile int*>(&sh.fail))
-        if (global_ns() - t0 > kTeamWaitNs) {
+    for (int k = lane; k < tm.T; k += 32) {
+      uint64_t got = ld_relaxed_u64(s + k);
+      TeamWait wait{global_ns(), got};
+      while ((uint32_t)(got >> 32) < want && !*reinterpret_cast<volatile int*>(&sh.fail)) {
+        if (team_wait_over(wait, global_ns(), got, sh.wait)) {
           set_status(tm.hdr, 5 /* CF_ERR_TIMEOUT */, tm.c);
           *reinterpret_cast<volatile int*>(&sh.fail) = 1;
         }
+        got = ld_relaxed_u64(s + k);
+      }
+    }
     __syncwarp();
   }
   __syncthreads();
@@ -382,7 +387,7 @@ __device__ __noinline__ void ring_slow_wait(TeamSh& sh, WsHeader* hdr, uint32_t 
   const uint64_t t0 = global_ns();
   for (uint32_t n = 0; !mbar_try(bar, parity); ++n) {
     if (*reinterpret_cast<volatile int*>(&sh.fail)) break;
-    if ((n & 255u) == 255u && global_ns() - t0 > kTeamWaitNs) {
+    if ((n & 255u) == 255u && global_ns() - t0 > sh.wait) {
       set_status(hdr, 5 /* CF_ERR_TIMEOUT */, -2);
       *reinterpret_cast<volatile int*>(&sh.fail) = 1;
       break;
@@ -439,7 +444,7 @@ __device__ __forceinline__ void ring_fill(const TeamStage& st, TeamSh& sh, WsHea
       spins = 0;
     } else {
       if (spins == 0) t0 = global_ns();
-      if ((++spins & 1023u) == 0u && global_ns() - t0 > kTeamWaitNs && lane == 0) {
+      if ((++spins & 1023u) == 0u && global_ns() - t0 > sh.wait && lane == 0) {
         set_status(hdr, 5 /* CF_ERR_TIMEOUT */, -3);
         *reinterpret_cast<volatile int*>(&sh.fail) = 1;
       }
@@ -1559,6 +1564,7 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
       if (lane == 0) best[i] = k;
     }
     team_sum(tm, sh, 0.f);
+    if (sh.fail) return 0.f;
     // the listed rows (every CTA finds the same ones): all rows down to a bin
     // of best values, at most kTop of them
     uint32_t v[kTeamRowsPer];
@@ -1657,6 +1663,7 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
       if (lane == 0) glen[s] = l;
     }
     team_sum(tm, sh, 0.f);
+    if (sh.fail) return 0.f;
     int made = 0;
     if (tm.c == 0) {
       uint32_t* key = reinterpret_cast<uint32_t*>(dead);  // the flags and candidates are done with
@@ -1720,7 +1727,8 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
         made = team_steps(sh, nl, need - matched, key, col, inv, idcol, len, sel, okey_out, olist, mrow, gdead);
     }
     const int got = (int)team_sum(tm, sh, t == 0 ? (float)made : 0.f);
-    if (got <= 0) break;  // a wait ran out
+    if (sh.fail) return 0.f;
+    if (got <= 0) break;  // (not reached: a phase takes the largest live entry)
     matched += got;
   }
   if (matched < need && tm.c == 0 && t == 0) set_status(tm.hdr, 6 /* CF_ERR_NUMERIC */, pidx);
@@ -1756,6 +1764,7 @@ __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const 
     return;
   }
   team_sum(tm, sh, 0.f);
+  if (sh.fail) return;
   if (tm.c == 0) {
     const Group cta{t, NT, 0, sh.redw, sh.redi};
     const float sc = greedy<int32_t>(cta, X, n_col, n_row, n_col, 0, ms, ms + n_row, ms + n_row + n_col, mo, cx.hdr,
@@ -2061,6 +2070,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
   }
   fence_async();
   const float tot = team_sum(tm, sh, ss);
+  if (sh.fail) return;
   float inv = 1.f;
   if (tot > 0.f) {
     inv = 1.0f / sqrtf(tot);
@@ -2081,6 +2091,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
     sk = team_far<NT>(tm, sh, TeamIter{eb, b0, b1, cx.alpha, inv, cbi, cx.K, cx.norm_mode}, g, ld, i0, i1,
                       region, nbr);
   }
+  if (sh.fail) return;
   // X_K in the caller's column order (rows of n_col): to the output, and for
   // the matching into b1 (the matching's lists then take E and b0)
   const float* Yk = cx.K == 0 ? eb : b0;
