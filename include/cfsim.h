@@ -104,8 +104,10 @@ typedef struct cf_params {
   int32_t match_mode; /* CF_MATCH_GREEDY (default) or CF_MATCH_OPTIMAL               */
   uint32_t flags;     /* CF_FLAG_*                                                */
   int32_t tune;       /* kernel configuration: 0 = built-in default (tune 1, with larger
-                         groups for small batches), else an id in
-                         [1, cf_num_tunes()] (cf_autotune picks one)              */
+                         groups and 512 threads for small batches, and the matching's
+                         steps in a second kernel, given room in the workspace, from 32
+                         pairs per SM on), else an id in [1, cf_num_tunes()]
+                         (cf_autotune picks one)                                  */
 } cf_params;
 
 /* One CFG on the host: blocks 0..n_blocks-1, edges src[e] -> dst[e] with weight
@@ -244,7 +246,8 @@ cf_status cf_topk_pairs(const int32_t* d_idx, int32_t Q, int32_t k, const int32_
 /* Workspace bytes cf_similarity / cf_match need for ANY list of P pairs of
  * these two packs (host copies): an upper bound of cf_similarity_ws_size for
  * pair lists that exist only on the device (e.g. from cf_topk_pairs).  It
- * sizes every pair as the two packs' largest CFGs. */
+ * sizes every pair as the two packs' largest CFGs; what tune 0 adds for many
+ * pairs is at most 2 GiB. */
 cf_status cf_similarity_ws_size_any(const void* h_pack_a, const void* h_pack_b, int32_t P, const cf_params* params,
                                     size_t* bytes);
 

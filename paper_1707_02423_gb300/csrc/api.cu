@@ -752,8 +752,14 @@ cf_status cf_similarity_ws_size_any(const void* h_pack_a, const void* h_pack_b, 
   const int sms = device_sm_count();
   const int64_t slots = std::min<int64_t>(P, 2 * (sms > 0 ? sms : 152));
   *bytes = ws_layout(P).fixed_bytes + (size_t)slots * global_slot_bytes(ha.max_blocks, hb.max_blocks);
-  if (params && decode_tune(params->tune).ranked == 3 && !(params->flags & CF_FLAG_PER_PAIR_LAUNCH))
-    *bytes += defer_bytes(P, (int64_t)P * ha.max_blocks * hb.max_blocks);
+  const Tune tn = call_tune(params, P);
+  if (params && tn.ranked == 3 && !(params->flags & CF_FLAG_PER_PAIR_LAUNCH)) {
+    const int64_t most = (int64_t)P * ha.max_blocks * hb.max_blocks;
+    if (!tn.defer_auto)
+      *bytes += defer_bytes(P, most);
+    else if (most >= kDeferCells * P)  // some lists may be large enough on average
+      *bytes += std::min(defer_bytes(P, most), kDeferMost);
+  }
   return ok();
 }
 
