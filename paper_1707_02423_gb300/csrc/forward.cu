@@ -110,6 +110,24 @@ __device__ __forceinline__ Geo make_geo(const Ctx& cx, int p, const ClassCfg& cc
   return g;
 }
 
+// The pair with its graphs' roles exchanged.
+__device__ __forceinline__ Geo swapped(const Geo& g) {
+  Geo s = g;
+  s.na = g.nb;
+  s.nb = g.na;
+  s.r_optr = g.c_optr;
+  s.r_iptr = g.c_iptr;
+  s.r_oadj = g.c_oadj;
+  s.r_iadj = g.c_iadj;
+  s.r_attr = g.c_attr;
+  s.c_optr = g.r_optr;
+  s.c_iptr = g.r_iptr;
+  s.c_oadj = g.r_oadj;
+  s.c_iadj = g.r_iadj;
+  s.c_attr = g.r_attr;
+  return s;
+}
+
 // Terms of an iteration of pair p, as the plan counts them.
 __device__ __forceinline__ int64_t pair_cost(const Ctx& cx, int p) {
   const int pa = __ldg(cx.pairs + 2 * p), pb = __ldg(cx.pairs + 2 * p + 1);

@@ -79,7 +79,8 @@ __device__ __forceinline__ PairFacts pair_facts(const PlanCtx& c, int p, const C
   int64_t cost = (int64_t)f.na * f.nb + 2 * (int64_t)ea * eb;
   // the global class is split over teams by cost: a CTA's shared memory also
   // limits the rows of its slab (about 2,000)
-  if (f.cls == kClassGlobal && cost < (int64_t)kTeamRowCost * f.na) cost = (int64_t)kTeamRowCost * f.na;
+  const int64_t rows = team_tr(f.na, f.nb) ? f.nb : f.na;
+  if (f.cls == kClassGlobal && cost < kTeamRowCost * rows) cost = kTeamRowCost * rows;
   f.bucket = cost_bucket(cost);
   return f;
 }

@@ -1750,7 +1750,7 @@ template <int NT>
 __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const Team& tm, TeamSh& sh, float* slot,
                                              const float* X, float* lists, unsigned char* region, int region_bytes) {
   const int t = threadIdx.x, n_row = g.na, n_col = g.nb;
-  float* rn = slot + 3 * (size_t)n_row * team_ld(n_col);
+  float* rn = slot + 3 * team_elems(n_row, n_col);
   int32_t* ms = reinterpret_cast<int32_t*>(rn + n_row + n_col);
   int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
   const GreedyForm form = greedy_form(n_row, n_col, NT, region_bytes);
@@ -1779,13 +1779,15 @@ __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const 
 // n_col rounded up to 8: bulk copies take multiples of 16 bytes), row and
 // column norms, matching state.  E holds the unscaled attribute term: Y_0 = E
 // with s_0 = 1 / |E|_F, and (1 - alpha) Ehat = (1 - alpha) / |E|_F E, so no
-// pass scales it.
+// pass scales it.  A tall pair's matrices are kept transposed up to X_K.
 template <int NT>
-__device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team& tm, TeamSh& sh, float* slot,
+__device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& given, const Team& tm, TeamSh& sh, float* slot,
                                         unsigned char* region, int region_bytes) {
   constexpr int NW = NT / 32, NC = kConsumers<NT>;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int n_row = g.na, n_col = g.nb;  // never transposed
+  const bool tr = team_tr(given.na, given.nb);
+  const Geo g = tr ? swapped(given) : given;
+  const int n_row = g.na, n_col = g.nb;
   const uint32_t ld = (uint32_t)team_ld(n_col), ld4 = 4 * ld;
   const size_t E = (size_t)n_row * ld;
   float* eb = slot;
@@ -2101,7 +2103,8 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
   for (int i = i0 + w; i < i1; i += NW)
     for (int p = lane; p < n_col; p += 32) {
       const float x = Yk[(size_t)i * ld + p] * sk;
-      const size_t to = (size_t)i * n_col + (staged ? cnat[p] : p);
+      const int j = staged ? cnat[p] : p;
+      const size_t to = tr ? (size_t)j * n_row + i : (size_t)i * n_col + j;
       if (xo) xo[to] = x;
       if (want) Xn[to] = x;
     }
@@ -2109,7 +2112,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& g, const Team&
     team_sum(tm, sh, 0.f);  // the slot is free for the next pair
     return;
   }
-  match_pair_t<NT>(cx, g, tm, sh, slot, Xn, eb, region, region_bytes);
+  match_pair_t<NT>(cx, given, tm, sh, slot, Xn, eb, region, region_bytes);
 }
 
 }  // namespace
