@@ -1282,6 +1282,97 @@ constexpr int kBins = 256;
 // neither the copy in (along a list) nor the steps (along an entry) conflict
 constexpr int kKeyPitch = kTop + 1, kColPitch = kTop + 2;
 
+// Writes a row's m chosen entries (up to kLen, in column order, at the front of
+// cand) in greedy order: each counts the ones before it.
+__device__ __forceinline__ void rank_list(uint2* cand, int m, uint2* out, int lane) {
+  // (c = lane + 32 q: the candidates of a block before block q come before
+  // c where equal, those of a block after it do not)
+  uint32_t* keys = reinterpret_cast<uint32_t*>(cand + kLen);  // past the chosen ones
+  for (int d = lane; d < ((m + 31) & ~31); d += 32) keys[d] = d < m ? cand[d].x : 0u;
+  __syncwarp();
+  for (int q = 0; 32 * q < m; ++q) {
+    const int c = lane + 32 * q;
+    const uint2 a = c < m ? cand[c] : make_uint2(0xffffffffu, 0u);
+    int rank = 0;
+    for (int b = 0; 32 * b < m; ++b) {
+      const uint4* kp = reinterpret_cast<const uint4*>(keys + 32 * b);
+      if (b != q) {
+        const uint32_t t = b < q ? a.x - 1u : a.x;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+          const uint4 k = kp[d];
+          rank += (k.x > t) + (k.y > t) + (k.z > t) + (k.w > t);
+        }
+      } else {
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+          const uint4 k = kp[d];
+          rank += (k.x > a.x - (uint32_t)(4 * d < lane)) + (k.y > a.x - (uint32_t)(4 * d + 1 < lane)) +
+                  (k.z > a.x - (uint32_t)(4 * d + 2 < lane)) + (k.w > a.x - (uint32_t)(4 * d + 3 < lane));
+        }
+      }
+    }
+    if (c < m) out[rank] = a;
+  }
+  __syncwarp();
+}
+
+// list_row where a row has too many candidates, or more than K entries of one
+// value: over the row, the key hi that at most K entries reach while more than K
+// reach the largest one below it, by halving between keys that occur; if few reach
+// hi, the first entries of that one as well.  bound: a key that more than K entries
+// reach, top: the largest.  (One entry after another over the row, 500 matrices of
+// 13 x 5,000 with three values took 5.5 ms, near rank one 0.5; now 0.7.  A function
+// of its own: in line it cost the other rows' lists 3 % of a call.)
+__device__ __noinline__ int list_row_far(const float* x, int n_col, const unsigned char* dead, int K, uint32_t bound,
+                                         uint32_t top, uint2* cand, uint2* out, int lane) {
+  uint32_t lo = bound, hi = top + 1u;
+  int gt = 0;
+  auto key_at = [&](int j) -> uint32_t {
+    const float v = j < n_col ? x[j] : 0.f;
+    return j < n_col && !dead[j] && v > -CUDART_INF_F ? okey(v) : 0u;
+  };
+  while (hi - lo > 1u && 4 * gt < 3 * K) {
+    const uint32_t mid = lo + (hi - lo) / 2;
+    uint32_t up = 0xffffffffu, down = 0u;
+    int c = 0;
+    for (int j0 = 0; j0 < n_col; j0 += 256) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t k = key_at(j0 + 32 * u + lane);
+        c += k >= mid;
+        up = k >= mid ? min(up, k) : up;
+        down = k >= mid ? down : max(down, k);
+      }
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c > K) {
+      lo = __reduce_min_sync(0xffffffffu, up);
+    } else {
+      hi = __reduce_max_sync(0xffffffffu, down) + 1u;
+      gt = c;
+    }
+  }
+  const int eq = 4 * gt < 3 * K ? K - gt : 0;  // (hi is lo + 1)
+  int m = 0, same = 0;
+  for (int j0 = 0; j0 < n_col; j0 += 256) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = j0 + 32 * u + lane;
+      const uint32_t k = key_at(j);
+      const unsigned lt = (1u << lane) - 1u, ms = __ballot_sync(0xffffffffu, k == lo);
+      const bool in = k >= hi || (k == lo && same + __popc(ms & lt) < eq);
+      const unsigned mt = __ballot_sync(0xffffffffu, in);
+      if (in) cand[m + __popc(mt & lt)] = make_uint2(k, (uint32_t)j);
+      m += __popc(mt);
+      same += __popc(ms);
+    }
+  }
+  __syncwarp();
+  rank_list(cand, m, out, lane);
+  return m;
+}
+
 // The list of one row: x = its entries, dead = column flags (shared memory),
 // cand = the warp's candidates.  Returns its length (bit 8: every live column
 // is in it).
@@ -1342,8 +1433,7 @@ __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigne
       }
     }
     if (cnt <= K) {
-      // the chosen ones to the front (candidates are in column order), then
-      // each counts the ones before it
+      // the chosen ones to the front (candidates are in column order)
       int m = 0;
       for (int d0 = 0; d0 < n; d0 += 32) {
         const uint2 a = d0 + lane < n ? cand[d0 + lane] : make_uint2(0u, 0u);
@@ -1352,58 +1442,11 @@ __device__ __forceinline__ int list_row(const float* x, int n_col, const unsigne
         m += __popc(in);
         __syncwarp();
       }
-      // (c = lane + 32 q: the candidates of a block before block q come before
-      // c where equal, those of a block after it do not)
-      uint32_t* keys = reinterpret_cast<uint32_t*>(cand + kLen);  // past the chosen ones
-      for (int d = lane; d < ((m + 31) & ~31); d += 32) keys[d] = d < m ? cand[d].x : 0u;
-      __syncwarp();
-      for (int q = 0; 32 * q < m; ++q) {
-        const int c = lane + 32 * q;
-        const uint2 a = c < m ? cand[c] : make_uint2(0xffffffffu, 0u);
-        int rank = 0;
-        for (int b = 0; 32 * b < m; ++b) {
-          const uint4* kp = reinterpret_cast<const uint4*>(keys + 32 * b);
-          if (b != q) {
-            const uint32_t t = b < q ? a.x - 1u : a.x;
-#pragma unroll
-            for (int d = 0; d < 8; ++d) {
-              const uint4 k = kp[d];
-              rank += (k.x > t) + (k.y > t) + (k.z > t) + (k.w > t);
-            }
-          } else {
-#pragma unroll
-            for (int d = 0; d < 8; ++d) {
-              const uint4 k = kp[d];
-              rank += (k.x > a.x - (uint32_t)(4 * d < lane)) + (k.y > a.x - (uint32_t)(4 * d + 1 < lane)) +
-                      (k.z > a.x - (uint32_t)(4 * d + 2 < lane)) + (k.w > a.x - (uint32_t)(4 * d + 3 < lane));
-            }
-          }
-        }
-        if (c < m) out[rank] = a;
-      }
-      __syncwarp();
+      rank_list(cand, m, out, lane);
       return m | (low == 0u && m == n ? 256 : 0);
     }
   }
-  // long runs of equal values: the best entries one after another
-  uint64_t prev = ~0ull;
-  int r = 0;
-  for (; r < K; ++r) {
-    uint64_t best = 0;
-    for (int j = lane; j < n_col; j += 32) {
-      const float v = x[j];
-      if (dead[j] || !(v > -CUDART_INF_F)) continue;
-      const uint64_t k = ((uint64_t)okey(v) << 32) | (uint32_t)~j;
-      if (k < prev && k > best) best = k;
-    }
-    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32));
-    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0u);
-    if (hi == 0u) break;
-    prev = ((uint64_t)hi << 32) | lo;
-    if (lane == 0) out[r] = make_uint2(hi, ~lo);
-  }
-  __syncwarp();
-  return r | (r < K ? 256 : 0);
+  return list_row_far(x, n_col, dead, K, bound, top, cand, out, lane);
 }
 
 // Step 3 of a phase, kTop threads (thread t: list t, row sel[t], rows
