@@ -1632,35 +1632,41 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     vmax = (uint32_t)(mm >> 32);
     if (vmax == 0u) break;  // no entry is left that can be taken
     vmin = ~(uint32_t)mm;
-    const int shift = max(0, 32 - __clz(vmax - vmin) - 8);
+    int shift = max(0, 32 - __clz(vmax - vmin) - 8), bin;
+    for (;;) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const uint32_t k = value(m);
-      if (k) atomicAdd(&bins[(vmax - k) >> shift], 1);
-    }
-    __syncthreads();
-    if (w == 0) {  // the last bin that keeps the count within kTop
-      int run = 0, last = -1;
-      for (int q0 = 0; q0 < kBins; q0 += 32) {
-        int c = bins[q0 + lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, c, o);
-          if (lane >= o) c += u;
-        }
-        c += run;
-        const unsigned ok = __ballot_sync(0xffffffffu, c <= kTop);
-        if (ok) last = q0 + 31 - __clz(ok);  // counts do not fall: a prefix of the lanes
-        run = __shfl_sync(0xffffffffu, c, 31);
-        if (ok != 0xffffffffu) break;
+      for (int m = 0; m < M; ++m) {
+        const uint32_t k = value(m), q = (vmax - k) >> shift;
+        if (k && q < (uint32_t)kBins) atomicAdd(&bins[q], 1);
       }
-      if (lane == 0) sh.bin = last;
+      __syncthreads();
+      if (w == 0) {  // the last bin that keeps the count within kTop
+        int run = 0, last = -1;
+        for (int q0 = 0; q0 < kBins; q0 += 32) {
+          int c = bins[q0 + lane];
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, c, o);
+            if (lane >= o) c += u;
+          }
+          c += run;
+          const unsigned ok = __ballot_sync(0xffffffffu, c <= kTop);
+          if (ok) last = q0 + 31 - __clz(ok);  // counts do not fall: a prefix of the lanes
+          run = __shfl_sync(0xffffffffu, c, 31);
+          if (ok != 0xffffffffu) break;
+        }
+        if (lane == 0) sh.bin = last;
+      }
+      __syncthreads();
+      bin = sh.bin;
+      if (bin >= 0 || shift == 0) break;
+      // the first bin alone holds more than kTop rows: its own range in bins
+      shift = max(0, shift - 8);
+      for (int q = t; q < kBins; q += NT) bins[q] = 0;
+      __syncthreads();
     }
-    __syncthreads();
-    const int bin = sh.bin;
-    // (the first bin alone may hold more than kTop rows, many of equal value:
-    // then the largest value's rows by index, up to kTop)
-    auto listed = [&](uint32_t k) { return k != 0u && (bin >= 0 ? (int)((vmax - k) >> shift) <= bin : k == vmax); };
+    // (more than kTop rows of the largest value: the first kTop of them by index)
+    auto listed = [&](uint32_t k) { return k != 0u && (bin >= 0 ? (vmax - k) >> shift <= (uint32_t)bin : k == vmax); };
     uint64_t below = 0;  // the best row that is not listed
 #pragma unroll
     for (int m = 0; m < M; ++m) {
