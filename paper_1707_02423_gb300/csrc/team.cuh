@@ -1588,7 +1588,37 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     int* bins = reinterpret_cast<int*>(rest);
     for (int q = t; q < kBins; q += NT) bins[q] = 0;
     __syncthreads();
-    for (int i = i0 + w; i < i1; i += NW) {
+    const int cw = ceil_div(n_col, 32), side = cw <= 8 ? 16 / cw : 0;
+    if (side) {  // short rows: as many of them as give 16 loads in flight
+      for (int i = i0 + w; i < i1; i += NW * side) {
+        const int mine = i + NW * lane;
+        const unsigned live = __ballot_sync(0xffffffffu, lane < side && mine < i1 && mrow[min(mine, i1 - 1)] < 0);
+        float v[16];
+#pragma unroll
+        for (int u = 0, r = 0, c = 0; u < 16; ++u) {
+          const int j = 32 * c + lane;
+          v[u] = (live >> r & 1u) && j < n_col ? X[(size_t)(i + NW * r) * n_col + j] : -CUDART_INF_F;
+          if (++c == cw) {
+            c = 0;
+            ++r;
+          }
+        }
+        uint32_t k = 0;
+#pragma unroll
+        for (int u = 0, r = 0, c = 0; u < 16; ++u) {
+          const int j = 32 * c + lane;
+          if (v[u] > -CUDART_INF_F && !dead[j]) k = max(k, okey(v[u]));
+          if (++c == cw) {
+            k = __reduce_max_sync(0xffffffffu, k);
+            if (lane == 0 && r < side && i + NW * r < i1) best[i + NW * r] = k;
+            k = 0;
+            c = 0;
+            ++r;
+          }
+        }
+      }
+    }
+    for (int i = i0 + w; !side && i < i1; i += NW) {
       uint32_t k = 0;
       if (mrow[i] < 0) {
         const float* x = X + (size_t)i * n_col;
