@@ -340,14 +340,18 @@ struct TeamTable {
 //     at 64 K, 102 at 128 K, 97 at 256 K, 318 at 512 K (no longer staged);
 //   - while the pairs leave CTAs free, a pair's share of them by its cells, down
 //     to kTeamMin entries, so that all pairs take about as long.
+// match: the matching of given matrices alone, by the share only.  It has no
+// iterates to keep in L2, and its steps, on one CTA of a team, are what a pair
+// takes: 152 pairs of 3,000 x 3,000 120 -> 51 ms,
+// of 5,200 x 5,200 1,515 -> 252.
 // cost = n_a n_b + 2 e_a e_b is about 3.65 n_a n_b for CFGs (1.15 edges per
 // block); total: the cost of all pairs of the class.
 constexpr int64_t kTeamEntries = 131072;
 constexpr int64_t kTeamMin = 1024;
 constexpr int kTeamRowCost = 320;  // cost counted per row at least
-CF_HD int team_level(int64_t cost, int64_t total, int n_cta) {
+CF_HD int team_level(int64_t cost, int64_t total, int n_cta, bool match = false) {
   const int64_t cells = cost * 20 / 73;
-  int64_t T = cells / kTeamEntries;
+  int64_t T = match ? 0 : cells / kTeamEntries;
   const int64_t most = cells / kTeamMin;
   int64_t share = (int64_t)((double)cost * n_cta / (double)total + 0.5);
   if (share > most) share = most;

@@ -80,7 +80,7 @@ __device__ __forceinline__ PairFacts pair_facts(const PlanCtx& c, int p, const C
   // the global class is split over teams by cost: a CTA's shared memory also
   // limits the rows of its slab (about 2,000)
   const int64_t rows = team_tr(f.na, f.nb) ? f.nb : f.na;
-  if (f.cls == kClassGlobal && cost < kTeamRowCost * rows) cost = kTeamRowCost * rows;
+  if (f.cls == kClassGlobal && cc.bwd != 2 && cost < kTeamRowCost * rows) cost = kTeamRowCost * rows;
   f.bucket = cost_bucket(cost);
   return f;
 }
@@ -173,7 +173,7 @@ __device__ __forceinline__ void queue_order(uint32_t* hist, uint32_t* n_class) {
 
 // Team levels of the global class (the queue's first): the queue position
 // each level ends at, from the class's counts (one thread; cnt: per bucket).
-__device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, int n_cta, uint32_t* lvl_end) {
+__device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, int n_cta, bool match, uint32_t* lvl_end) {
   // a bucket's middle cost: 2 to 3, or 3 to 4, times 2^(b / 2)
   auto mid = [](int b) { return (int64_t)((b & 1) ? 7 : 5) << (b / 2) >> 1; };
   int64_t total = 0;
@@ -183,7 +183,7 @@ __device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, in
   int level = 0;
   for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
     if (cnt[b] == 0) continue;
-    level = max(level, team_level(mid(b), total, n_cta));
+    level = max(level, team_level(mid(b), total, n_cta, match));
     seen += cnt[b];
 #pragma unroll
     for (int L = 0; L < kTeamLevels; ++L)
@@ -267,7 +267,8 @@ __global__ void __launch_bounds__(kPlanSmallNT) plan_small_kernel(CallArgs a, Cl
     c.m_off[c.P] = tm;
     defer_area(c.hdr, a, cc.ranked, tx, s_class[kClassGlobal] + s_class[kClassCluster],
                (size_t)*reinterpret_cast<volatile uint64_t*>(&c.hdr->slot_need));
-    if (s_class[kClassGlobal] > 0) team_levels(s_glob, s_class[kClassGlobal], a.n_cta, c.hdr->team.lvl_end);
+    if (s_class[kClassGlobal] > 0)
+      team_levels(s_glob, s_class[kClassGlobal], a.n_cta, cc.bwd == 2, c.hdr->team.lvl_end);
   }
 }
 
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_count_kernel(CallArgs a, Cl
 
 constexpr int kScanNT = 512;
 
-__global__ void __launch_bounds__(kScanNT) plan_scan_kernel(CallArgs a, int ranked) {
+__global__ void __launch_bounds__(kScanNT) plan_scan_kernel(CallArgs a, int ranked, bool match) {
   __shared__ uint32_t hist[kSlots], s_class[kNumClasses], s_glob[kBuckets];
   PlanCtx c = plan_ctx(a);
   const int t = threadIdx.x;
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(kScanNT) plan_scan_kernel(CallArgs a, int rank
     c.m_off[c.P] = tm;
     defer_area(c.hdr, a, ranked, tx, s_class[kClassGlobal] + s_class[kClassCluster], (size_t)c.hdr->slot_need);
     // (the levels' table takes the histogram's place)
-    team_levels(s_glob, s_class[kClassGlobal], a.n_cta, c.hdr->team.lvl_end);
+    team_levels(s_glob, s_class[kClassGlobal], a.n_cta, match, c.hdr->team.lvl_end);
   }
 }
 
@@ -372,7 +373,7 @@ cudaError_t launch_plan(const CallArgs& args, const ClassCfg& cc, cudaStream_t s
   if (z != cudaSuccess) return z;
   WsLayout L = ws_layout(a.P);
   plan_count_kernel<<<L.plan_blocks, kPlanThreads, 0, s>>>(a, cc);
-  plan_scan_kernel<<<1, kScanNT, 0, s>>>(a, cc.ranked);
+  plan_scan_kernel<<<1, kScanNT, 0, s>>>(a, cc.ranked, cc.bwd == 2);
   plan_scatter_kernel<<<L.plan_blocks, kPlanThreads, 0, s>>>(a, cc);
   return cudaGetLastError();
 }
