@@ -168,7 +168,8 @@ __device__ __forceinline__ int64_t pair_cost(const Ctx& cx, int p) {
 // the bound is reached first (NaN in X) the status word gets CF_ERR_NUMERIC.
 // tg: n_col entries (round stamps, values up to min(n_row, n_col)).
 // Returns the score on every thread; writes match[n_a] if given.
-template <class IdxT, class Grp>
+// U: a lane's loads in flight in a rescan (matrices in memory: 8).
+template <class IdxT, int U = 1, class Grp>
 __device__ __forceinline__ float greedy(const Grp& grp, const float* X, int ld, int n_row, int n_col, int tr,
                                         IdxT* rb, IdxT* cb, IdxT* tg, int32_t* mo, WsHeader* hdr, int pidx) {
   const int t = grp.rank, G = grp.size, lane = t & 31, w = grp.warp(), NW = grp.nwarps();
@@ -189,14 +190,20 @@ __device__ __forceinline__ float greedy(const Grp& grp, const float* X, int ld, 
         float bv = -CUDART_INF_F;
         int bi = 0x7fffffff;
         const float* xr = X + (size_t)r * ld;
-        for (int c = lane; c < n_col; c += 32)
-          if (cb[c] > (IdxT)-3) {
-            const float x = xr[c];
-            if (x > bv) {
-              bv = x;
-              bi = c;
-            }
+        for (int c0 = lane; c0 < n_col; c0 += 32 * U) {
+          float x[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int c = c0 + 32 * u;
+            x[u] = c < n_col && cb[c] > (IdxT)-3 ? xr[c] : -CUDART_INF_F;
           }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (x[u] > bv) {
+              bv = x[u];
+              bi = c0 + 32 * u;
+            }
+        }
         warp_argmax(bv, bi);
         v = bi == 0x7fffffff ? -1 : bi;
         if (lane == 0) rb[r] = (IdxT)v;
@@ -210,14 +217,20 @@ __device__ __forceinline__ float greedy(const Grp& grp, const float* X, int ld, 
       if (!(v == -2 || (v >= 0 && rb[v] <= (IdxT)-3))) continue;
       float bv = -CUDART_INF_F;
       int bi = 0x7fffffff;
-      for (int r = lane; r < n_row; r += 32)
-        if (rb[r] > (IdxT)-3) {
-          const float x = X[(size_t)r * ld + c];
-          if (x > bv) {
-            bv = x;
-            bi = r;
-          }
+      for (int r0 = lane; r0 < n_row; r0 += 32 * U) {
+        float x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int r = r0 + 32 * u;
+          x[u] = r < n_row && rb[r] > (IdxT)-3 ? X[(size_t)r * ld + c] : -CUDART_INF_F;
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (x[u] > bv) {
+            bv = x[u];
+            bi = r0 + 32 * u;
+          }
+      }
       warp_argmax(bv, bi);
       if (lane == 0) cb[c] = bi == 0x7fffffff ? (IdxT)-1 : (IdxT)bi;
     }
@@ -922,6 +935,40 @@ __device__ __noinline__ float match_steps(int lane, bool by_row, int nl, int len
   return warp_sum(sc);
 }
 
+// Whether rounds of locally dominant entries take many entries each: of 32
+// elements spread over all, how many are the best of the list that they are the
+// best in.  In a random matrix that is half of them or more, in an X_K of 80
+// blocks and more at most a sixteenth (60 pairs); ten is the line.  (1,000
+// matrices of 200 x 200, steps / rounds: random 3.11 / 0.91 ms, near rank one 4.0 /
+// 20; 3,000 of 120 x 120 random 1.99 / 0.82.)  With fewer than 80 elements the steps
+// are about as fast on random ones too: 5,000 of 60 x 60 0.68 ms, 0.88 by rounds.
+constexpr int kRoundsLen = 80;
+__device__ __forceinline__ bool rounds_pay(const Group& grp, const uint32_t* key, int nl, int len, int ld) {
+  const int lane = grp.rank & 31;
+  int own = 0;
+  for (int s = grp.warp(); s < 32; s += grp.nwarps()) {
+    const int e = s * len / 32;
+    uint32_t k = 0u;
+    int at = 0;
+    for (int l = lane; l < nl; l += 32) {
+      const uint32_t q = key[e * ld + l];
+      if (q > k) {
+        k = q;
+        at = l;
+      }
+    }
+    const uint32_t best = __reduce_max_sync(0xffffffffu, k);
+    at = __reduce_min_sync(0xffffffffu, k == best ? at : 0x7fffffff);
+    bool less = false;
+    for (int q = lane; q < len; q += 32) {
+      const uint32_t x = key[q * ld + at];
+      less |= x > best || (x == best && q < e);
+    }
+    own += !__any_sync(0xffffffffu, less);
+  }
+  return grp.sum_i(lane == 0 ? own : 0, 0) >= 10;
+}
+
 // a5-a6 on the caller's matrix (cf_match): the sequential greedy on ranked
 // lists, as the forward does, on a group of the pair's size.  Lists run along
 // the shorter side and their keys lie [element][list], so that the lanes of a
@@ -938,11 +985,12 @@ __device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const 
   const bool by_row = nb <= na;
   const int nl = by_row ? na : nb, len = by_row ? nb : na;
   float sc = 0.f;
-  if (nl <= kSeqMaxLists) {
-    const int ld = nl | 1;
-    uint32_t* key = reinterpret_cast<uint32_t*>(region);
-    unsigned char* rk = region + align_up(4 * (size_t)len * ld, 16);
-    unsigned char* dead = rk + nl * len;
+  bool rounds = nl > kSeqMaxLists;
+  const int ld = nl | 1;
+  uint32_t* key = reinterpret_cast<uint32_t*>(region);
+  unsigned char* rk = region + align_up(4 * (size_t)len * ld, 16);
+  unsigned char* dead = rk + nl * len;
+  if (!rounds) {
     for (int i0 = t; i0 < tot; i0 += 8 * G) {
       float v[8];
 #pragma unroll
@@ -957,6 +1005,9 @@ __device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const 
       for (int i = t; i < na; i += G) mo[i] = -1;
     for (int e = t; e < len; e += G) dead[e] = 0;
     grp.sync();
+    if (len >= kRoundsLen) rounds = rounds_pay(grp, key, nl, len, ld);
+  }
+  if (!rounds) {
     // rank of element e in list l: elements with a larger key, or an equal key
     // and a smaller index (keys are >= 1)
     for (int idx = t; idx < tot; idx += G) {
@@ -982,7 +1033,7 @@ __device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const 
       else
         sc = match_steps<8>(t, by_row, nl, len, ld, key, rk, dead, mo, cx.hdr, g.p);
     }
-  } else {
+  } else {  // (from kRoundsLen elements on the state fits in the ranks' place)
     float* Xs = reinterpret_cast<float*>(region);
     int16_t* ms = reinterpret_cast<int16_t*>(region + align_up(4 * (size_t)tot, 16));
     for (int idx = t; idx < tot; idx += G) Xs[idx] = __ldg(src + idx);
@@ -1221,7 +1272,7 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
       __syncthreads();
       if ((uint32_t)sh.n0 >= n) return;
       const Geo g = make_geo(cx, (int)cx.queue[sh.n0], cc);
-      const float sc = greedy<int16_t>(cta, cx.X_in + cx.x_off[g.p], g.nb, g.na, g.nb, 0, ms, ms + g.na,
+      const float sc = greedy<int16_t, 8>(cta, cx.X_in + cx.x_off[g.p], g.nb, g.na, g.nb, 0, ms, ms + g.na,
                                        ms + g.na + g.nb, cx.match ? cx.match + cx.m_off[g.p] : nullptr, cx.hdr, g.p);
       if (cx.scores && t == 0) cx.scores[g.p] = sc;
     }
@@ -1291,7 +1342,7 @@ __global__ void __launch_bounds__(kTeamNT, 1) fwd_team_kernel(CallArgs a, ClassC
       float* slot = reinterpret_cast<float*>(align_up(reinterpret_cast<size_t>(cx.scratch + si * need), 16));
       const Geo g = make_geo(cx, (int)cx.queue[pos], cc);
       if constexpr (kMatch)
-        match_pair_t<kTeamNT>(cx, g, tm, sh, slot, cx.X_in + cx.x_off[g.p], slot, smem, kTeamSmem);
+        match_pair_t<kTeamNT, true>(cx, g, tm, sh, slot, cx.X_in + cx.x_off[g.p], slot, smem, kTeamSmem);
       else
         run_pair_t<kTeamNT>(cx, g, tm, sh, slot, smem, kTeamSmem);
       if (sh.fail) return;

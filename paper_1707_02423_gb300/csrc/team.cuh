@@ -1558,9 +1558,9 @@ __device__ __forceinline__ GreedyForm greedy_form(int n_row, int n_col, int NT, 
 // and visible to the team.  lists: scratch of 8 n_row n_col bytes; ms: n_row
 // ints (row matches), then n_col bytes (column flags); best: n_row ints.  Ends
 // with a team barrier.  Returns the score on every thread.
-// (5,200 x 5,200 given, near rank one: 11.5 ms in the wide form, 5,000 x 5,200 8.9
-// ms in the other; one CTA with greedy(), the team waiting, 7.6 s.  152 such pairs:
-// 1.52 s, against 12.4 s with a CTA per pair.)
+// (5,200 x 5,200 given, near rank one: 11.3 ms in the wide form, 5,000 x 5,200 9.2
+// ms in the other; one CTA with greedy(), the team waiting, 7.6 s.  152 such pairs,
+// a CTA each: 0.25 s in phases, 12.4 s with greedy().)
 template <int NT, bool kWide>
 __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const float* X, int n_row, int n_col,
                                           uint2* lists, int32_t* ms, uint32_t* best, unsigned char* region,
@@ -1822,17 +1822,69 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
   return team_sum(tm, sh, sc);
 }
 
+// rounds_pay for a matrix in memory, by the CTA: of 16 lines of the shorter side,
+// a warp each, four or more are the best of their best entry's other line; of
+// four, three where that side is short (16 would be the whole matrix, and in a
+// random one nearly all of them are).
+template <int NT>
+__device__ __forceinline__ bool rounds_pay_t(TeamSh& sh, const float* X, int n_row, int n_col) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  static_assert(NT >= 512, "a warp per line");
+  const int S = min(n_row, n_col), L = max(n_row, n_col);
+  const size_t sa = n_row <= n_col ? n_col : 1, sb = n_row <= n_col ? 1 : n_col;  // from line to line, along a line
+  auto key_at = [&](int q, int e) -> uint32_t {
+    const float v = q < S && e < L ? X[q * sa + e * sb] : -CUDART_INF_F;
+    return v > -CUDART_INF_F ? okey(v) : 0u;
+  };
+  const int lines = S < 32 ? 4 : 16;
+  if (w < lines) {
+    const int line = (int)((int64_t)S * w / lines);
+    uint32_t k = 0u;
+    int at = 0;
+    for (int e0 = lane; e0 < L; e0 += 256) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t q = key_at(line, e0 + 32 * u);
+        if (q > k) {
+          k = q;
+          at = e0 + 32 * u;
+        }
+      }
+    }
+    const uint32_t best = __reduce_max_sync(0xffffffffu, k);
+    at = __reduce_min_sync(0xffffffffu, k == best ? at : 0x7fffffff);
+    bool less = best == 0u;
+    for (int q0 = lane; q0 < S; q0 += 256) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int q = q0 + 32 * u;
+        const uint32_t x = key_at(q, at);
+        less |= x > best || (x == best && q < line);
+      }
+    }
+    less = __any_sync(0xffffffffu, less);
+    if (lane == 0) sh.redi[w] = !less;
+  }
+  __syncthreads();
+  const int pay = __popc(__ballot_sync(0xffffffffu, lane < lines && sh.redi[lane]));
+  __syncthreads();
+  return pay >= (S < 32 ? 3 : 4);
+}
+
 // The matching of a team's pair: X row-major n_row x n_col, written by the team
 // (or the caller's); lists: scratch of two matrices; the slot's state arrays.
-// Ends with a team barrier.
-template <int NT>
+// Ends with a team barrier.  kGiven: the caller's matrix, which need not be close
+// to rank one; one CTA then takes it by rounds where they pay (a team's phases
+// are the faster all the same).
+template <int NT, bool kGiven>
 __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const Team& tm, TeamSh& sh, float* slot,
                                              const float* X, float* lists, unsigned char* region, int region_bytes) {
   const int t = threadIdx.x, n_row = g.na, n_col = g.nb;
   float* rn = slot + 3 * team_elems(n_row, n_col);
   int32_t* ms = reinterpret_cast<int32_t*>(rn + n_row + n_col);
   int32_t* mo = cx.match ? cx.match + cx.m_off[g.p] : nullptr;
-  const GreedyForm form = greedy_form(n_row, n_col, NT, region_bytes);
+  GreedyForm form = greedy_form(n_row, n_col, NT, region_bytes);
+  if (kGiven && tm.T == 1 && form != kGreedySmall && rounds_pay_t<NT>(sh, X, n_row, n_col)) form = kGreedySmall;
   if (form != kGreedySmall) {
     uint2* ls = reinterpret_cast<uint2*>(lists);
     uint32_t* best = reinterpret_cast<uint32_t*>(rn);
@@ -1846,8 +1898,9 @@ __device__ __forceinline__ void match_pair_t(const Ctx& cx, const Geo& g, const 
   if (sh.fail) return;
   if (tm.c == 0) {
     const Group cta{t, NT, 0, sh.redw, sh.redi};
-    const float sc = greedy<int32_t>(cta, X, n_col, n_row, n_col, 0, ms, ms + n_row, ms + n_row + n_col, mo, cx.hdr,
-                                     g.p);
+    int16_t* st = reinterpret_cast<int16_t*>(region);
+    const float sc = greedy<int16_t, 8>(cta, X, n_col, n_row, n_col, 0, st, st + n_row, st + n_row + n_col, mo, cx.hdr,
+                                        g.p);
     if (cx.scores && t == 0) cx.scores[g.p] = sc;
     __syncthreads();  // team_sum takes redw, which greedy's last sum was read from
   }
@@ -2191,7 +2244,7 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& given, const T
     team_sum(tm, sh, 0.f);  // the slot is free for the next pair
     return;
   }
-  match_pair_t<NT>(cx, given, tm, sh, slot, Xn, eb, region, region_bytes);
+  match_pair_t<NT, false>(cx, given, tm, sh, slot, Xn, eb, region, region_bytes);
 }
 
 }  // namespace
