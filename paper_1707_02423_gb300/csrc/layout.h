@@ -342,18 +342,22 @@ struct TeamTable {
 //     to kTeamMin entries, so that all pairs take about as long.
 // match: the matching of given matrices alone, by the share only.  It has no
 // iterates to keep in L2, and its steps, on one CTA of a team, are what a pair
-// takes: 152 pairs of 3,000 x 3,000 120 -> 51 ms,
-// of 5,200 x 5,200 1,515 -> 252.
+// takes: 152 pairs of 3,000 x 3,000 120 -> 51 ms, of 5,200 x 5,200 1,515 -> 252.
+// even: all pairs cost about the same.  A share is then rounded down: rounded up,
+// the pairs outnumber the teams and a few of them make a second wave (100 pairs of
+// 40 x 600 1.15 ms on teams of two, 0.78 alone; of 150 x 150 1.50 and 1.06).  Among
+// pairs of many sizes the small ones fill the gaps, and rounding down loses (100
+// pairs of 150-700 blocks 4.5 -> 6.5 ms).
 // cost = n_a n_b + 2 e_a e_b is about 3.65 n_a n_b for CFGs (1.15 edges per
 // block); total: the cost of all pairs of the class.
 constexpr int64_t kTeamEntries = 131072;
 constexpr int64_t kTeamMin = 1024;
 constexpr int kTeamRowCost = 320;  // cost counted per row at least
-CF_HD int team_level(int64_t cost, int64_t total, int n_cta, bool match = false) {
+CF_HD int team_level(int64_t cost, int64_t total, int n_cta, bool match = false, bool even = false) {
   const int64_t cells = cost * 20 / 73;
   int64_t T = match ? 0 : cells / kTeamEntries;
   const int64_t most = cells / kTeamMin;
-  int64_t share = (int64_t)((double)cost * n_cta / (double)total + 0.5);
+  int64_t share = (int64_t)((double)cost * n_cta / (double)total + (even ? 0. : 0.5));
   if (share > most) share = most;
   if (T < share) T = share;
   if (T < 1) T = 1;

@@ -177,13 +177,21 @@ __device__ __forceinline__ void team_levels(const uint32_t* cnt, uint32_t ng, in
   // a bucket's middle cost: 2 to 3, or 3 to 4, times 2^(b / 2)
   auto mid = [](int b) { return (int64_t)((b & 1) ? 7 : 5) << (b / 2) >> 1; };
   int64_t total = 0;
-  for (int b = 0; b < kBuckets; ++b) total += cnt[b] * mid(b);
+  int lo = kBuckets, hi = -1;
+  for (int b = 0; b < kBuckets; ++b) {
+    total += cnt[b] * mid(b);
+    if (cnt[b]) {
+      lo = min(lo, b);
+      hi = b;
+    }
+  }
+  const bool even = hi - lo <= 1;  // within an octave
   uint32_t seen = 0;
   uint32_t end[kTeamLevels] = {};
   int level = 0;
   for (int b = kBuckets - 1; b >= 0 && seen < ng; --b) {
     if (cnt[b] == 0) continue;
-    level = max(level, team_level(mid(b), total, n_cta, match));
+    level = max(level, team_level(mid(b), total, n_cta, match, even));
     seen += cnt[b];
 #pragma unroll
     for (int L = 0; L < kTeamLevels; ++L)
