@@ -1,5 +1,5 @@
 """Greedy matching in phases of matrices with short rows, whose best values a warp
-finds several rows at a time: one chunk of 32 columns up to eight, and nine."""
+finds several rows at a time: up to two chunks of 32 columns, and beyond."""
 import numpy as np
 import pytest
 import torch
