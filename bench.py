@@ -274,7 +274,7 @@ def measured_peaks():
 
 # The sources the forward kernels are built from; a committed profile counts
 # only while their hash is the one it was taken with.
-KERNEL_SOURCES = ("forward.cu", "iterate.cuh", "layout.h", "device_common.cuh")
+KERNEL_SOURCES = ("forward.cu", "team.cuh", "iterate.cuh", "layout.h", "device_common.cuh")
 
 
 def kernel_sources_sha256(csrc: str) -> str:

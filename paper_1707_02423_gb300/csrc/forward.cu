@@ -977,7 +977,7 @@ __device__ __forceinline__ bool rounds_pay(const Group& grp, const uint32_t* key
 // an entry instead of the forward's 12, so that more pairs are at work on an SM.
 // What bounds it is the chain of steps, one warp's per pair.  (4,950 pairs of
 // 8-120 blocks, the kernel: one CTA per pair and rounds of rescans 1.61 ms, the
-// forward's three buffers 0.535; the call 1.81 ms, 0.76 and, as here, 0.57.)
+// forward's three buffers 0.535; the call 1.81 ms, 0.76 and, as here, 0.53.)
 __device__ __forceinline__ void match_pair_s(const Ctx& cx, const Geo& g, const Group& grp, unsigned char* region) {
   const int t = grp.rank, G = grp.size, na = g.na, nb = g.nb, tot = na * nb;
   const float* src = cx.X_in + cx.x_off[g.p];
@@ -1838,7 +1838,7 @@ cudaError_t launch_forward(const CallArgs& a, int variant, bool per_pair, cudaSt
     const cudaError_t e = launch_team<false>(a, fwd_class_cfg(variant, a.min_cls, a.ranked, a.cluster), s);
     if (e != cudaSuccess) return e;
   }
-  if (!per_pair && a.cluster >= 2) {  // the cluster tier first: its pairs are the largest
+  if (!per_pair && a.cluster >= 2) {  // then the cluster tier
     const cudaError_t e = variant == 1   ? launch_cluster<512>(a, s)
                           : variant == 2 ? launch_cluster<768>(a, s)
                                          : launch_cluster<1024>(a, s);

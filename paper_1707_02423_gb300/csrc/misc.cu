@@ -43,10 +43,11 @@ constexpr int kTopkCand = 256 + 2 * kTopkMax;  // candidates, 256 + 2 k of them 
 // ~column), all different, so ties go to the smaller column and the result is
 // exact and deterministic.  Thread t owns the columns t + NT m.
 //   1  the best key of each group of threads (a warp or a part of one, so that
-//      there are at least 1.5 k groups); the k-th best of these is a bound
+//      there are at least 1.5 k groups, as far as the threads go: 1,024 groups
+//      at most, 256 up to 2,048 columns); the k-th best of these is a bound
 //      that at least k elements reach, in random order little more than k;
 //   2  the elements that reach the bound are collected and ranked by counting.
-// Two reads of the row and four barriers for any k.  A row whose best elements
+// Two reads of the row and three barriers for any k.  A row whose best elements
 // crowd into few groups has too many candidates: it goes by rounds, each the
 // block's maximum of the threads' best keys, after which the warp of the
 // winner's thread finds that thread's next best.

@@ -63,7 +63,6 @@ __host__ __device__ __forceinline__ void team_split(int nch, int NC, int& CH, in
 // What the sweep needs of a pair (in shared memory).  Addresses of shared
 // memory are 32-bit (ld.shared, not generic loads).
 struct TeamStage {
-  const uint16_t* cnat;   // column position -> column
   const int4* cA;         // per column in order of kind: {4 out 0, weight, 4 in 0, weight} (positions), in the
                           // ring's place until the warps have read them
   const int4* brow;       // per busy row of the whole row graph: its out- and in-ranges in redge
@@ -1589,7 +1588,9 @@ __device__ __noinline__ float greedy_team(const Team& tm, TeamSh& sh, const floa
     for (int q = t; q < kBins; q += NT) bins[q] = 0;
     __syncthreads();
     const int cw = ceil_div(n_col, 32), side = cw <= 2 ? 16 / cw : 0;
-    if (side) {  // short rows: as many of them as give 16 loads in flight (up to eight chunks: 2 % slower at 200 columns)
+    // short rows: as many of them as give 16 loads in flight (for up to eight
+    // chunks of columns in place of two, 2 % slower at 200 columns)
+    if (side) {
       for (int i = i0 + w; i < i1; i += NW * side) {
         const int mine = i + NW * lane;
         const unsigned live = __ballot_sync(0xffffffffu, lane < side && mine < i1 && mrow[min(mine, i1 - 1)] < 0);
@@ -2111,7 +2112,6 @@ __device__ __noinline__ void run_pair_t(const Ctx& cx, const Geo& given, const T
       const int li = i1 > i0 ? i1 - 1 : i0;  // rows of the slab that are not busy
       const uint32_t m = m0[li >> 5], bit = 1u << (li & 31);
       st.nr = i1 > i0 ? li - ((int)p0[li >> 5] + __popc(m & (bit - 1u))) - base + (m & bit ? 0 : 1) : 0;
-      st.cnat = cnat;
       st.cA = cA;
       st.cb = (uint32_t)__cvta_generic_to_shared(cB) - 16u * (uint32_t)ps;
       st.brow = brow;
